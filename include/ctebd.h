@@ -231,7 +231,8 @@ int mps_load_device(ctebd_mps* mps, const int* chi, const void* const* sites,
 /* Per-split log of the last step() / truncate_split: rows of 12 doubles
    (q0, k, bond, m, n, r, f, W, sketched, eigen-dimension, rank before the
    chi_max cap, rank hint, Jacobi sweeps of the first pass, Jacobi sweeps of
-   the FP32 refinement pass) -- 14 doubles per row.  *n_rows receives the row count; up to cap rows
+   the FP32 refinement pass; both 0 where the direct solver ran) -- 14 doubles
+   per row.  *n_rows receives the row count; up to cap rows
    are written. */
 int mps_split_log(const ctebd_mps* mps, double* rows, int cap, int* n_rows);
 
@@ -312,7 +313,9 @@ int ctebd_set_sweep_graphs(int mode);
 /* Sweep cap of the Jacobi eigen-solves of the split (not in the paper; the
    solver of this implementation), process-wide, 1..1000 (default 60: the
    first pass takes about 10 sweeps at width 2048, the refinement pass up to
-   about 20 on steep spectra).  A solve whose problems still make significant
+   about 20 on steep spectra).  Full splits of the handle calls use a direct
+   solver without sweeps unless the cap is below 12 or the tensor-core policy
+   is 2; the Jacobi solver then takes them, with this cap.  A solve whose problems still make significant
    rotations after n sweeps makes step / truncate_split / split2_noalloc return
    CTEBD_ERR_NUMERIC (the state's sites of that iteration are then
    undefined).  Errors: ARG. */

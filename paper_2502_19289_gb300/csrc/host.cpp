@@ -382,11 +382,13 @@ struct Work {
 // ---------------------------------------------------------------------------
 enum KernelKind {
   KK_GEMM_MERGE, KK_GEMM_U, KK_GEMM_GRAM, KK_GEMM_PROJ, KK_EIG_INIT, KK_EIG_INNER, KK_EIG_APPLY,
-  KK_COLNORM, KK_SELECT, KK_GATHER, KK_ONEQ, KK_AMP, KK_GEMM_SKETCH, KK_CHOL, KK_MLP, KK_COUNT
+  KK_COLNORM, KK_SELECT, KK_GATHER, KK_ONEQ, KK_AMP, KK_GEMM_SKETCH, KK_CHOL, KK_MLP,
+  KK_BIDIAG, KK_TRIDIAG, KK_BACK, KK_COUNT
 };
 static const char* kKindNames[KK_COUNT] = {
   "gemm_merge", "gemm_apply_u", "gemm_gram", "gemm_project", "eig_init", "eig_inner", "eig_apply",
-  "colnorm", "select", "gather", "apply_1q", "amplitude", "gemm_sketch", "cholqr", "mlp_forward"};
+  "colnorm", "select", "gather", "apply_1q", "amplitude", "gemm_sketch", "cholqr", "mlp_forward",
+  "bidiag", "tridiag_eig", "back_transform"};
 
 struct Prof {
   bool on = false;
@@ -468,6 +470,9 @@ struct ctebd_mps {
   size_t eig_scr_cap = 0;          // in doubles
   unsigned char* pack_scr = nullptr;   // packed tensor-core GEMM operands (high-water)
   size_t pack_cap = 0;                 // in bytes
+  unsigned char* dir_scr = nullptr;    // direct solver: barriers, exchange buffers, per-problem scratch (high-water)
+  size_t dir_cap = 0;                  // in bytes
+  int n_sm = 0;
   cudaStream_t side = nullptr;     // second branch of the device-side sweep graphs
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   void* arena = nullptr;
@@ -524,7 +529,14 @@ extern "C" int mps_create(const ctebd_config* cfg, void* cuda_stream, ctebd_mps*
   m->lam.assign(m->n + 1, nullptr);
   int rc = m->stage.init(8 << 20, m->stream);
   if (rc) { mps_destroy(m); return rc; }
-  if (cudaMallocHost(&m->h_res, 16 * sizeof(double) * 4096) != cudaSuccess) { mps_destroy(m); return fail(CTEBD_ERR_OOM, "pinned"); }
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (cudaDeviceGetAttribute(&m->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || m->n_sm < 1) {
+    mps_destroy(m);
+    return fail(CTEBD_ERR_CUDA, "mps_create: device attributes");
+  }
+  // 16 doubles per problem, then the copy of the kernels' wait flag
+  if (cudaMallocHost(&m->h_res, 16 * sizeof(double) * (4096 + 1)) != cudaSuccess) { mps_destroy(m); return fail(CTEBD_ERR_OOM, "pinned"); }
   m->h_res_cap = 4096;
   std::vector<double> one(1, 1.0);
   for (int b = 0; b <= m->n; b++) {
@@ -565,6 +577,7 @@ extern "C" int mps_destroy(ctebd_mps* m) {
   if (m->tc_err) cudaFree(m->tc_err);
   if (m->eig_scr) cudaFree(m->eig_scr);
   if (m->pack_scr) cudaFree(m->pack_scr);
+  if (m->dir_scr) cudaFree(m->dir_scr);
   if (m->h_res) cudaFreeHost(m->h_res);
   m->stage.release();
   m->prof.release();
@@ -1280,6 +1293,8 @@ static int level_eig(ctebd_mps* m, std::vector<Work>& ws, const Level& L, const 
   return CTEBD_OK;
 }
 
+static int check_tc_flag(ctebd_mps* m);
+
 // Rfull = Mbar V (bufB, m x ne), rho = weighted column norms, truncation
 // select (with the total weight ||M||^2 for sketched problems); results to host
 static int level_project_select(ctebd_mps* m, std::vector<Work>& ws, const Level& L,
@@ -1359,11 +1374,110 @@ static int level_project_select(ctebd_mps* m, std::vector<Work>& ws, const Level
                            m->stream));
   }
   // results land at the level-local index a (h_res[16 a .. 16 a + 15])
+  int* h_flag = reinterpret_cast<int*>(m->h_res + 16 * m->h_res_cap);
+  *h_flag = 0;
   if (L.act.size() > m->h_res_cap) return fail(CTEBD_ERR_ARG, "too many clusters");
   for (int a : sel)
     CUDA_TRY(cudaMemcpyAsync(m->h_res + 16 * a, ws[L.act[a]].res, 16 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+  if (m->tc_err) CUDA_TRY(cudaMemcpyAsync(h_flag, m->tc_err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
   CUDA_TRY(cudaStreamSynchronize(m->stream));
   m->stage.reset();
+  if (*h_flag) return check_tc_flag(m);
+  return CTEBD_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Direct solver (svd_direct.cu): V of every problem of the selection from the
+// weighted split matrix itself.
+// ---------------------------------------------------------------------------
+static int ensure_dir_scratch(ctebd_mps* m, size_t n) {
+  if (n <= m->dir_cap) return CTEBD_OK;
+  CUDA_TRY(cudaStreamSynchronize(m->stream));
+  if (m->dir_scr) CUDA_TRY(cudaFree(m->dir_scr));
+  m->dir_scr = nullptr;
+  m->dir_cap = 0;
+  const size_t want = n + n / 4;
+  if (cudaMalloc(&m->dir_scr, want) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(CTEBD_ERR_OOM, "direct solver scratch of " + std::to_string(want >> 20) + " MiB");
+  }
+  m->dir_cap = want;
+  return CTEBD_OK;
+}
+
+template <typename R>
+static int level_direct(ctebd_mps* m, std::vector<Work>& ws, const Level& L, const std::vector<int>& sel) {
+  if (sel.empty()) return CTEBD_OK;
+  // classes of similar width, one bidiagonalisation launch each
+  auto bucket = [&](int a) {
+    int b = 64;
+    while (b < L.nn[a]) b <<= 1;
+    return b;
+  };
+  std::vector<int> order(sel);
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return bucket(x) > bucket(y); });
+  const int na = (int)order.size();
+  struct Class { int first, count, m, n; };
+  std::vector<Class> cls;
+  int max_n = 0;
+  for (int i = 0; i < na; i++) {
+    const int a = order[i];
+    if (cls.empty() || bucket(order[cls.back().first]) != bucket(a)) cls.push_back({i, 0, 0, 0});
+    Class& c = cls.back();
+    c.count++;
+    c.m = std::max(c.m, L.mm[a]);
+    c.n = std::max(c.n, L.nn[a]);
+    max_n = std::max(max_n, L.nn[a]);
+  }
+  const size_t bar_bytes = round_up(sizeof(unsigned) * m->n_sm, 256);
+  size_t xchg = 0, dbl = 0;
+  for (const Class& c : cls) xchg = std::max(xchg, round_up(dir_xchg_bytes<R>(c.m, c.n, c.count, m->n_sm), 256));
+  for (int a : order) dbl += dir_scratch_doubles(L.nn[a]);
+  TRY(ensure_dir_scratch(m, bar_bytes + xchg + dbl * sizeof(double)));
+  TRY(ensure_tc_err(m));
+  unsigned* bars = reinterpret_cast<unsigned*>(m->dir_scr);
+  void* xbuf = m->dir_scr + bar_bytes;
+  double* p = reinterpret_cast<double*>(m->dir_scr + bar_bytes + xchg);
+  std::vector<DirProb> dp(na);
+  double fl_b = 0, fl_t = 0, fl_v = 0;
+  for (const Class& c : cls)
+    for (int i = c.first; i < c.first + c.count; i++) {
+      const int a = order[i];
+      Work& w = ws[L.act[a]];
+      DirProb& q = dp[i];
+      const int n = L.nn[a];
+      q.M = w.bufA; q.lam = m->lam[w.q0]; q.m = L.mm[a]; q.n = n; q.shift = L.shift[a]; q.depth = dir_depth(n);
+      q.A = w.bufB;
+      q.VR = w.G;
+      q.Q0 = w.W;
+      q.Q1 = static_cast<R*>(w.W) + (size_t)n * n;
+      q.S = w.V;      // free until the back-transformation writes V
+      q.V = w.V; q.ldv = L.vld[a];
+      q.xld = c.n;
+      dir_carve(q, p);
+      p += dir_scratch_doubles(n);
+      const double mm = q.m, nd = n, k = std::min(q.m, n);
+      fl_b += 16.0 * (mm * nd * k - (mm + nd) * k * k / 2 + k * k * k / 3);
+      fl_t += 8.0 / 3.0 * nd * nd * nd;
+      fl_v += 8.0 * nd * nd * nd;
+    }
+  const DirProb* dd;
+  TRY(m->stage.push(dp.data(), dp.size(), &dd));
+  {
+    ProfScope ps(m->prof, m->stream, KK_BIDIAG, fl_b, 0);
+    m->prof.launches[KK_BIDIAG] += (double)cls.size() - 1;
+    for (const Class& c : cls)
+      CUDA_TRY(launch_dir_bidiag<R>(dd + c.first, c.count, c.m, c.n, xbuf, bars, m->tc_err, m->n_sm, m->stream));
+  }
+  {
+    ProfScope ps(m->prof, m->stream, KK_TRIDIAG, fl_t, 0);
+    int launches = 0;
+    CUDA_TRY(launch_dir_tridiag<R>(dd, na, max_n, &launches, m->stream));
+    m->prof.launches[KK_TRIDIAG] += launches - 1;
+  }
+  ProfScope ps(m->prof, m->stream, KK_BACK, fl_v, 0);
+  m->prof.launches[KK_BACK] += 1;
+  CUDA_TRY(launch_dir_back<R>(dd, na, max_n, m->stream));
   return CTEBD_OK;
 }
 
@@ -1513,10 +1627,28 @@ static int level_sketch(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
   return CTEBD_OK;
 }
 
+// Full splits take the direct solver; the Jacobi solver keeps sketched splits,
+// runs with a sweep cap too low for it to be of use (a caller that lowers the
+// cap wants the error of a solve that does not converge), and the policy that
+// forces every product onto the tensor cores.
+// 12 sweeps are what the Jacobi first pass takes at most on the widths it is
+// used for; 4096 is the widest split of the ABI.
+constexpr int kDirectMinCap = 12, kDirectMaxWidth = 4096;
+static bool use_direct(int n) {
+  return g_max_sweeps >= kDirectMinCap && g_tc_mode != 2 && n <= kDirectMaxWidth;
+}
+
 // pass 1 (+ FP32 pass 2) for a selection: Gram of Z, eigen-solve, V, weights, select
-static int level_solve(ctebd_mps* m, std::vector<Work>& ws, Level& L, const std::vector<int>& sel) {
-  if (sel.empty()) return CTEBD_OK;
+static int level_solve(ctebd_mps* m, std::vector<Work>& ws, Level& L, const std::vector<int>& all) {
+  if (all.empty()) return CTEBD_OK;
   const bool f64 = m->fp64;
+  std::vector<int> sel, direct;
+  for (int a : all) (!L.sk[a] && use_direct(L.nn[a]) ? direct : sel).push_back(a);
+  if (!direct.empty()) {
+    TRY(f64 ? level_direct<double>(m, ws, L, direct) : level_direct<float>(m, ws, L, direct));
+    TRY(level_project_select(m, ws, L, direct));
+  }
+  if (sel.empty()) return CTEBD_OK;
   std::vector<const void*> Z;
   std::vector<void*> accV;
   for (int a : sel) {

@@ -59,6 +59,43 @@ struct EigProb {
                        // (rounded up to even) indices; 0: all 2 JB
 };
 
+// One problem of the direct solver (svd_direct.cu): the right singular vectors
+// of diag(lam) M (m x n, row-major, row r weighted by lam[r >> shift]).
+struct DirProb {
+  const void* M;
+  const double* lam;
+  int m, n, shift, depth;   // depth: dir_depth(n)
+  void* A;         // m x n working copy (used when the rows exceed shared memory)
+  void* VR;        // n x n: right reflectors, row k = v_k
+  void* Q0;        // n x n real, run precision: eigenvectors of B^T B (ping)
+  void* Q1;        // pong
+  void* S;         // n x n real: eigenvectors of a merge's rank-one update
+  void* V;         // out: n x n right singular vectors, leading dimension ldv
+  int ldv;
+  int xld;         // row length of the exchange buffers (largest n of the class)
+  // per-problem scratch (dir_carve): panel factors, reflector scalars, B,
+  // eigenvalues, first / last eigenvector rows, merge work
+  void* T;
+  void* tau;
+  double *dd, *ee, *D, *fr, *lr, *F, *Lr, *dl, *zl, *zh, *tauq, *rc, *rsn, *rho;
+  int *org, *pos, *gcol, *perm, *rcol, *rcol2, *meta;
+};
+int dir_depth(int n);
+size_t dir_scratch_doubles(int n);
+void dir_carve(DirProb& q, double* p);
+// Golub-Kahan step of a class of problems (largest m and n of the class);
+// exchange scratch of dir_xchg_bytes, n_sm barrier counters, and a flag that a
+// bounded wait sets when it runs out
+template <typename R>
+size_t dir_xchg_bytes(int m, int n, int count, int n_sm);
+template <typename R>
+cudaError_t launch_dir_bidiag(const DirProb* probs, int count, int m, int n, void* xchg, unsigned* bars, int* err,
+                              int n_sm, cudaStream_t s);
+template <typename R>
+cudaError_t launch_dir_tridiag(const DirProb* probs, int count, int max_n, int* launches, cudaStream_t s);
+template <typename R>
+cudaError_t launch_dir_back(const DirProb* probs, int count, int max_n, cudaStream_t s);
+
 // Per-problem truncation inputs/outputs of one split level.
 struct SelProb {
   const double* rho;   // n weighted column norms
