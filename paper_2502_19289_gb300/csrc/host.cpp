@@ -470,7 +470,7 @@ struct ctebd_mps {
   size_t eig_scr_cap = 0;          // in doubles
   unsigned char* pack_scr = nullptr;   // packed tensor-core GEMM operands (high-water)
   size_t pack_cap = 0;                 // in bytes
-  unsigned char* dir_scr = nullptr;    // direct solver: barriers, exchange buffers, per-problem scratch (high-water)
+  unsigned char* dir_scr = nullptr;    // direct solver: exchange buffers, per-problem scratch (high-water)
   size_t dir_cap = 0;                  // in bytes
   int n_sm = 0;
   cudaStream_t side = nullptr;     // second branch of the device-side sweep graphs
@@ -1429,15 +1429,13 @@ static int level_direct(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
     c.n = std::max(c.n, L.nn[a]);
     max_n = std::max(max_n, L.nn[a]);
   }
-  const size_t bar_bytes = round_up(sizeof(unsigned) * m->n_sm, 256);
   size_t xchg = 0, dbl = 0;
   for (const Class& c : cls) xchg = std::max(xchg, round_up(dir_xchg_bytes<R>(c.m, c.n, c.count, m->n_sm), 256));
   for (int a : order) dbl += dir_scratch_doubles(L.nn[a]);
-  TRY(ensure_dir_scratch(m, bar_bytes + xchg + dbl * sizeof(double)));
+  TRY(ensure_dir_scratch(m, xchg + dbl * sizeof(double)));
   TRY(ensure_tc_err(m));
-  unsigned* bars = reinterpret_cast<unsigned*>(m->dir_scr);
-  void* xbuf = m->dir_scr + bar_bytes;
-  double* p = reinterpret_cast<double*>(m->dir_scr + bar_bytes + xchg);
+  void* xbuf = m->dir_scr;
+  double* p = reinterpret_cast<double*>(m->dir_scr + xchg);
   std::vector<DirProb> dp(na);
   double fl_b = 0, fl_t = 0, fl_v = 0;
   for (const Class& c : cls)
@@ -1467,7 +1465,7 @@ static int level_direct(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
     ProfScope ps(m->prof, m->stream, KK_BIDIAG, fl_b, 0);
     m->prof.launches[KK_BIDIAG] += (double)cls.size() - 1;
     for (const Class& c : cls)
-      CUDA_TRY(launch_dir_bidiag<R>(dd + c.first, c.count, c.m, c.n, xbuf, bars, m->tc_err, m->n_sm, m->stream));
+      CUDA_TRY(launch_dir_bidiag<R>(dd + c.first, c.count, c.m, c.n, xbuf, m->tc_err, m->n_sm, m->stream));
   }
   {
     ProfScope ps(m->prof, m->stream, KK_TRIDIAG, fl_t, 0);

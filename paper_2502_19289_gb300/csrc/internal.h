@@ -84,13 +84,13 @@ int dir_depth(int n);
 size_t dir_scratch_doubles(int n);
 void dir_carve(DirProb& q, double* p);
 // Golub-Kahan step of a class of problems (largest m and n of the class);
-// exchange scratch of dir_xchg_bytes, n_sm barrier counters, and a flag that a
+// exchange scratch of dir_xchg_bytes (16-byte aligned), and a flag that a
 // bounded wait sets when it runs out
 template <typename R>
 size_t dir_xchg_bytes(int m, int n, int count, int n_sm);
 template <typename R>
-cudaError_t launch_dir_bidiag(const DirProb* probs, int count, int m, int n, void* xchg, unsigned* bars, int* err,
-                              int n_sm, cudaStream_t s);
+cudaError_t launch_dir_bidiag(const DirProb* probs, int count, int m, int n, void* xchg, int* err, int n_sm,
+                              cudaStream_t s);
 template <typename R>
 cudaError_t launch_dir_tridiag(const DirProb* probs, int count, int max_n, int* launches, cudaStream_t s);
 template <typename R>

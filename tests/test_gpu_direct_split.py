@@ -81,7 +81,8 @@ def _unitary(rng):
 
 # (chi_L, chi_mid, chi_R): the split matrix is 2 chi_L x 2 chi_R
 SHAPES = [(1, 1, 1), (1, 2, 4), (2, 4, 4), (4, 5, 5), (5, 9, 16), (16, 16, 17), (32, 32, 32), (33, 40, 33),
-          (64, 64, 64), (65, 70, 65), (128, 128, 31), (31, 62, 100), (100, 128, 128), (129, 129, 129)]
+          (64, 64, 64), (65, 70, 65), (128, 128, 31), (31, 62, 100), (100, 128, 128), (129, 129, 129),
+          (300, 310, 290)]
 
 
 @pytest.mark.parametrize("prec", ["FP32", "FP64"])
