@@ -2070,25 +2070,35 @@ extern "C" int amplitude(const ctebd_mps* mc, const uint8_t* bits, double* re, d
   if (!m || !bits || !re || !im) return fail(CTEBD_ERR_ARG, "amplitude: null argument");
   int cmax = 1;
   for (int c : m->chi) cmax = std::max(cmax, c);
-  double2 *va = nullptr, *vb = nullptr;
-  CUDA_TRY(cudaMallocAsync(&va, sizeof(double2) * cmax, m->stream));
-  CUDA_TRY(cudaMallocAsync(&vb, sizeof(double2) * cmax, m->stream));
-  const double one[2] = {1.0, 0.0};
-  CUDA_TRY(cudaMemcpyAsync(va, one, sizeof(one), cudaMemcpyHostToDevice, m->stream));
+  std::vector<AmpSite> sites(m->n);
+  double fl = 0;
   for (int q = 0; q < m->n; q++) {
     if (bits[q] > 1) return fail(CTEBD_ERR_ARG, "amplitude: bits must be 0/1");
-    ProfScope ps(m->prof, m->stream, KK_AMP, 8.0 * m->chi[q] * m->chi[q + 1], (double)m->chi[q] * m->chi[q + 1] * m->esz);
-    CUDA_TRY(m->fp64 ? launch_amp_step<double>(va, vb, m->site[q], m->chi[q], m->chi[q + 1], bits[q], m->stream)
-                     : launch_amp_step<float>(va, vb, m->site[q], m->chi[q], m->chi[q + 1], bits[q], m->stream));
-    std::swap(va, vb);
+    sites[q] = {m->site[q], m->chi[q], m->chi[q + 1], bits[q]};
+    fl += 8.0 * m->chi[q] * m->chi[q + 1];
   }
-  double out[2];
-  CUDA_TRY(cudaMemcpyAsync(out, va, sizeof(out), cudaMemcpyDeviceToHost, m->stream));
-  CUDA_TRY(cudaFreeAsync(va, m->stream));
-  CUDA_TRY(cudaFreeAsync(vb, m->stream));
+  const size_t bytes = amp_scratch_bytes(cmax);
+  TRY(ensure_dir_scratch(m, bytes));
+  TRY(ensure_tc_err(m));
+  double2* out = reinterpret_cast<double2*>(m->dir_scr + bytes) - 1;
+  const AmpSite* ds;
+  m->stage.reset();   // every call has waited for the stream before it returned
+  TRY(m->stage.push(sites.data(), sites.size(), &ds));
+  const int ctas = amp_ctas(cmax, m->n_sm), mid = m->chi[m->n / 2];
+  int* h_flag = reinterpret_cast<int*>(m->h_res + 16 * m->h_res_cap);
+  *h_flag = 0;
+  {
+    ProfScope ps(m->prof, m->stream, KK_AMP, fl, fl / 8 * m->esz);
+    m->prof.launches[KK_AMP] += 1;
+    CUDA_TRY(m->fp64 ? launch_amplitude<double>(ds, m->n, mid, cmax, ctas, m->dir_scr, out, m->tc_err, m->stream)
+                     : launch_amplitude<float>(ds, m->n, mid, cmax, ctas, m->dir_scr, out, m->tc_err, m->stream));
+  }
+  CUDA_TRY(cudaMemcpyAsync(m->h_res, out, sizeof(double2), cudaMemcpyDeviceToHost, m->stream));
+  CUDA_TRY(cudaMemcpyAsync(h_flag, m->tc_err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
   CUDA_TRY(cudaStreamSynchronize(m->stream));
-  *re = out[0];
-  *im = out[1];
+  if (*h_flag) return check_tc_flag(m);
+  *re = m->h_res[0];
+  *im = m->h_res[1];
   return CTEBD_OK;
 }
 

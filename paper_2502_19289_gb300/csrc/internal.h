@@ -77,7 +77,8 @@ struct DirProb {
   // eigenvalues, first / last eigenvector rows, merge work
   void* T;
   void* tau;
-  double *dd, *ee, *D, *fr, *lr, *F, *Lr, *dl, *zl, *zh, *tauq, *rc, *rsn, *rho;
+  double *dd, *ee, *scale;
+  void *D, *fr, *lr, *F, *Lr, *dl, *zl, *zh, *tauq, *rc, *rsn, *rho;   // FP64 or FP32 pairs
   int *org, *pos, *gcol, *perm, *rcol, *rcol2, *meta;
 };
 int dir_depth(int n);
@@ -239,9 +240,20 @@ cudaError_t launch_gather(const GatherProb* d_probs, int n_probs, long long max_
 template <typename R>
 cudaError_t launch_apply_1q(void* const* d_sites, const int* d_cl, const int* d_cr,
                             const double* d_u, int n_sites, long long max_elems, cudaStream_t s);
+// One site of an amplitude: the chi_l x chi_r slice of its bit value.
+struct AmpSite {
+  const void* S;
+  int cl, cr, bit;
+};
+// <bits|psi> over n sites (out: one complex128): left and right halves of the
+// chain by amp_ctas(max_chi, n_sm) CTAs each; scratch of amp_scratch_bytes
+// (16-byte aligned; its last 16 bytes can hold out), and the flag that a
+// bounded wait sets when it runs out; mid_chi: the bond left of site n / 2
+int amp_ctas(int max_chi, int n_sm);
+size_t amp_scratch_bytes(int max_chi);
 template <typename R>
-cudaError_t launch_amp_step(const void* v_in, void* v_out, const void* site, int cl, int cr,
-                            int bit, cudaStream_t s);
+cudaError_t launch_amplitude(const AmpSite* d_sites, int n, int mid_chi, int max_chi, int ctas, unsigned char* scratch,
+                             double2* out, int* err, cudaStream_t s);
 template <typename R>
 cudaError_t launch_convert_from_c128(const double* src, void* dst, long long n, cudaStream_t s);
 template <typename R>

@@ -1248,33 +1248,6 @@ template cudaError_t launch_apply_1q<double>(void* const*, const int*, const int
                                              int, long long, cudaStream_t);
 
 template <typename R>
-__global__ void k_amp_step(const double2* __restrict__ vin, double2* __restrict__ vout,
-                           const void* __restrict__ site, int cl, int cr, int bit) {
-  using CT = typename C2<R>::T;
-  const CT* S = (const CT*)site;
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= cr) return;
-  double2 acc = make_double2(0, 0);
-  for (int a = 0; a < cl; a++) {
-    const CT s = S[((long long)a * 2 + bit) * cr + b];
-    const double2 v = vin[a];
-    acc.x += v.x * (double)s.x - v.y * (double)s.y;
-    acc.y += v.x * (double)s.y + v.y * (double)s.x;
-  }
-  vout[b] = acc;
-}
-
-template <typename R>
-cudaError_t launch_amp_step(const void* v_in, void* v_out, const void* site, int cl, int cr,
-                            int bit, cudaStream_t s) {
-  k_amp_step<R><<<(cr + 127) / 128, 128, 0, s>>>((const double2*)v_in, (double2*)v_out, site, cl,
-                                                 cr, bit);
-  return cudaGetLastError();
-}
-template cudaError_t launch_amp_step<float>(const void*, void*, const void*, int, int, int, cudaStream_t);
-template cudaError_t launch_amp_step<double>(const void*, void*, const void*, int, int, int, cudaStream_t);
-
-template <typename R>
 __global__ void k_from_c128(const double* __restrict__ src, void* __restrict__ dst, long long n) {
   using CT = typename C2<R>::T;
   CT* d = (CT*)dst;

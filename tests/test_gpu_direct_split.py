@@ -25,7 +25,7 @@ def _site(rng, a, b):
     return g.reshape(a, 2, b) if a <= 2 * b else (g / np.linalg.norm(g)).reshape(a, 2, b)
 
 
-def _state(rng, shapes, dtype):
+def _state(rng, shapes, dtype, decades=4.0):
     """Sites of two-site blocks (a, b, c) side by side, joined by bonds of 1."""
     chis, sites = [1], []
     for a, b, c in shapes:
@@ -34,7 +34,7 @@ def _state(rng, shapes, dtype):
             chis.append(y)
     lams = []
     for c in chis:
-        w = np.sort(rng.exponential(1.0, c) * 10.0 ** (-4.0 * np.arange(c) / c))[::-1]
+        w = np.sort(rng.exponential(1.0, c) * 10.0 ** (-decades * np.arange(c) / c))[::-1]
         lams.append(np.sqrt(w / w.sum()))
     return np.array(chis, dtype=np.int32), sites, lams
 
@@ -112,6 +112,16 @@ def test_direct_split_rank_deficient(rank, prec):
     chis, sites, lams = _state(rng, [(40, rank, 40)], np.complex64 if prec == "FP32" else np.complex128)
     lams[1] = np.full(40, 1 / np.sqrt(40))
     _check(lib(), chis, sites, lams, [1], [np.eye(4, dtype=np.complex128)], prec, 80, 0.0)
+
+
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+@pytest.mark.parametrize("decades", [8.0, 16.0])
+def test_direct_split_steep_wide(decades, prec):
+    """Fewer rows than columns and a steep spectrum: behind the rank, the bidiagonal ends in rounding
+    noise whose squares lie below FP32's range."""
+    rng = np.random.default_rng(int(decades))
+    chis, sites, lams = _state(rng, [(96, 98, 100)], np.complex64 if prec == "FP32" else np.complex128, decades)
+    _check(lib(), chis, sites, lams, [1], [_unitary(rng)], prec, 200, 1e-9)
 
 
 def test_direct_split_larger_than_shared_memory():
