@@ -192,13 +192,13 @@ int apply_cluster(ctebd_mps* mps, const ctebd_cluster* c, const double* U);
    k-1 truncated SVDs (right to left), truncation rule of Sec. II.B (chi_max
    and the relative discarded-weight cutoff eta), per-split fidelity f_j of
    Eq. 4 written to f_out[k-1] (may be NULL), product accumulated (Eq. 5).
-   Errors: STATE (nothing pending), CUDA, NUMERIC. */
+   Errors: STATE (nothing pending), CUDA, NUMERIC, TIMEOUT. */
 int truncate_split(ctebd_mps* mps, const ctebd_cluster* c, double* f_out);
 
 /* All clusters of one iteration, batched: every phase is one launch over all
    n clusters.  U[i]: host pointer to cluster i's unitary.  f_out: per-split
    fidelities, cluster by cluster (sum of k_i - 1 entries), may be NULL.
-   Clusters must be disjoint.  Errors: ARG, CUDA, NUMERIC. */
+   Clusters must be disjoint.  Errors: ARG, CUDA, NUMERIC, TIMEOUT. */
 int step(ctebd_mps* mps, const ctebd_cluster* c, int n, const double* const* U, double* f_out);
 
 /* Eq. 5: product of all per-split fidelities so far (FP64). */
@@ -370,7 +370,8 @@ int ctebd_measure_fma(int repeats, double* tflops_best, double* tflops_mean, int
    returning, so it cannot be called while that stream is being captured.
    Every call shares the array and leaves the previous call's data in it;
    calls that overlap on the GPU (other streams or threads) race on it.
-   Errors: ARG, CUDA, NUMERIC. */
+   Errors: ARG, CUDA, NUMERIC, TIMEOUT (such a race, or a bounded wait between
+   the CTAs of one launch that ran out). */
 int split2_noalloc(const void* theta, const double* lam_l, int chi_l, int chi_r, int chi_max,
                    double cutoff, void* site_l_out, void* site_r_out, double* lam_out,
                    int* r_out, double* f_out, void* cuda_stream);

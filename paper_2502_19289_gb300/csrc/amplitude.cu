@@ -19,7 +19,8 @@ namespace ctebd {
 
 namespace {
 
-constexpr int kAmpThreads = 256, kAmpAhead = 16;   // values of a site read ahead, per thread
+// four warps: one per FP64 unit of an SM
+constexpr int kAmpThreads = 128, kAmpAhead = 16;   // values of a site read ahead, per thread
 
 template <typename R> struct C2;
 template <> struct C2<float> { using T = float2; };
@@ -41,93 +42,109 @@ __global__ void __launch_bounds__(kAmpThreads, 1)
   if (tid == 0) { vs[0] = make_double2(1.0, 0.0); bad = 0; }
   // slice of a site: outputs [o0, o0 + no) of this CTA, `len` terms each;
   // thread -> output oi, terms t0, t0 + nt, ...
-  int o0 = 0, no = 0, len = 0, oi = 0, t0 = 0, nt = 1;
-  long long so = 0, st = 0;                                 // strides of an output and of a term
-  const CT* S = nullptr;
-  CT ahead[kAmpAhead];
-  auto open_site = [&](int k) {
-    const AmpSite a = sites[half == 0 ? k : n - 1 - k];
-    const int outs = half == 0 ? a.cr : a.cl;
-    len = half == 0 ? a.cl : a.cr;
-    const int per = (outs + G - 1) / G;
-    o0 = c * per;
-    no = max(0, min(per, outs - o0));
-    int p2 = 1;
-    while (p2 < per && p2 < kAmpThreads) p2 <<= 1;
-    nt = kAmpThreads / p2;
+  struct Slice {
+    int outs, o0, no, len, oi, t0, nt;
+    long long so, st;                                       // strides of an output and of a term
+    const CT* S;
+  };
+  auto site_at = [&](int k) { return sites[half == 0 ? k : n - 1 - k]; };
+  auto open_site = [&](const AmpSite& a, Slice& z, CT (&ahead)[kAmpAhead]) {
+    z.outs = half == 0 ? a.cr : a.cl;
+    z.len = half == 0 ? a.cl : a.cr;
+    const int per = G > 1 ? (z.outs + G - 1) / G : z.outs;
+    z.o0 = c * per;
+    z.no = max(0, min(per, z.outs - z.o0));
+    int lg = 0;                                             // threads per output: a power of two
+    while ((1 << lg) < per && (1 << lg) < kAmpThreads) lg++;
+    const int p2 = 1 << lg;
+    z.nt = kAmpThreads >> lg;
     // neighbouring threads read neighbouring elements of a row
-    oi = half == 0 ? tid % p2 : tid / nt;
-    t0 = half == 0 ? tid / p2 : tid % nt;
-    so = half == 0 ? 1 : 2LL * a.cr;
-    st = half == 0 ? 2LL * a.cr : 1;
-    S = reinterpret_cast<const CT*>(a.S) + (long long)a.bit * a.cr;
+    z.oi = half == 0 ? tid & (p2 - 1) : tid / z.nt;
+    z.t0 = half == 0 ? tid >> lg : tid & (z.nt - 1);
+    z.so = half == 0 ? 1 : 2LL * a.cr;
+    z.st = half == 0 ? 2LL * a.cr : 1;
+    z.S = reinterpret_cast<const CT*>(a.S) + (long long)a.bit * a.cr;
 #pragma unroll
     for (int i = 0; i < kAmpAhead; i++) {
-      const int t = t0 + i * nt;
-      if (oi < no && t < len) ahead[i] = S[(o0 + oi) * so + t * st];
+      const int t = z.t0 + i * z.nt;
+      if (z.oi < z.no && t < z.len) ahead[i] = z.S[(z.o0 + z.oi) * z.so + t * z.st];
     }
-    return outs;
   };
-  int outs = count > 0 ? open_site(0) : 0;
+  // a site's values are on their way while the site before it is worked on,
+  // its description one site earlier
+  Slice cur{}, nxt{};
+  CT now[kAmpAhead], ahead[kAmpAhead];
+  AmpSite desc{};
+  if (count > 0) open_site(site_at(0), cur, now);
+  if (count > 1) desc = site_at(1);
   __syncthreads();
   for (int k = 0; k < count; k++) {
     const unsigned seq = k + 1;
     unsigned char* buf = ex + (size_t)(seq & 1u) * max_chi * SB;
-    const int p2 = kAmpThreads / nt;
-    for (int ob = 0; ob < no; ob += p2) {                   // one turn unless a lone CTA has more outputs than threads
+    const bool more = k + 1 < count;
+    if (more) open_site(desc, nxt, ahead);
+    if (k + 2 < count) desc = site_at(k + 2);
+    const int p2 = kAmpThreads / cur.nt;
+    for (int ob = 0; ob < cur.no; ob += p2) {               // one turn unless a lone CTA has more outputs than threads
       double2 acc = make_double2(0, 0);
       auto term = [&](int t, CT s) {
         const double2 v = vs[t];
         acc.x = fma(v.x, (double)s.x, acc.x); acc.x = fma(-v.y, (double)s.y, acc.x);
         acc.y = fma(v.x, (double)s.y, acc.y); acc.y = fma(v.y, (double)s.x, acc.y);
       };
-      if (ob + oi < no) {
+      if (ob + cur.oi < cur.no) {
         if (ob == 0) {
 #pragma unroll
-          for (int i = 0; i < kAmpAhead; i++)
-            if (t0 + i * nt < len) term(t0 + i * nt, ahead[i]);
+          for (int i = 0; i < kAmpAhead; i++) {
+            if (i * cur.nt >= cur.len) break;               // for all threads alike
+            if (cur.t0 + i * cur.nt < cur.len) term(cur.t0 + i * cur.nt, now[i]);
+          }
         }
-        for (int t = t0 + (ob == 0 ? kAmpAhead * nt : 0); t < len; t += nt) term(t, S[(o0 + ob + oi) * so + t * st]);
+        for (int t = cur.t0 + (ob == 0 ? kAmpAhead * cur.nt : 0); t < cur.len; t += cur.nt)
+          term(t, cur.S[(cur.o0 + ob + cur.oi) * cur.so + t * cur.st]);
       }
       // sum over the nt threads of an output
-      const int at = oi * nt + t0;
+      const int at = cur.oi * cur.nt + cur.t0;
       red[at] = acc;
       __syncthreads();
-      for (int s = nt >> 1; s > 0; s >>= 1) {
-        if (t0 < s) {
+      for (int s = cur.nt >> 1; s > 0; s >>= 1) {
+        if (cur.t0 < s) {
           red[at].x += red[at + s].x;
           red[at].y += red[at + s].y;
         }
         __syncthreads();
       }
-      if (tid < p2 && ob + tid < no) {
-        const double2 v = red[tid * nt];
-        if (G > 1) Slot<double2>::put(buf + (size_t)(o0 + ob + tid) * SB, v, seq);
+      if (tid < p2 && ob + tid < cur.no) {
+        const double2 v = red[tid * cur.nt];
+        if (G > 1) Slot<double2>::put(buf + (size_t)(cur.o0 + ob + tid) * SB, v, seq);
         else vs[max_chi + kAmpThreads + ob + tid] = v;      // the next vector (a lone CTA)
       }
       __syncthreads();
     }
-    const int len_next = outs;
-    if (k + 1 < count) outs = open_site(k + 1);
     if (G > 1) {
       // A CTA without a slice of the next site skips this vector.  (One that
       // has a slice holds up the vector after the next, so the slots it still
       // has to read are not written again before.)
-      const bool need = k + 1 < count ? no > 0 : c == 0;
-      for (int j = tid; need && j < len_next; j += kAmpThreads) {
+      const bool need = more ? nxt.no > 0 : c == 0;
+      for (int j = tid; need && j < cur.outs; j += kAmpThreads) {
         const unsigned char* ad[1] = {buf + (size_t)j * SB};
         double2 v[1];
         if (!poll(ad, seq, v, err)) bad = 1;
         vs[j] = v[0];
       }
     } else {
-      for (int j = tid; j < len_next; j += kAmpThreads) vs[j] = vs[max_chi + kAmpThreads + j];
+      for (int j = tid; j < cur.outs; j += kAmpThreads) vs[j] = vs[max_chi + kAmpThreads + j];
     }
     __syncthreads();
     if (bad) return;
+    if (more) {
+      cur = nxt;
+#pragma unroll
+      for (int i = 0; i < kAmpAhead; i++) now[i] = ahead[i];
+    }
   }
   if (c == 0) {
-    const int m = count > 0 ? outs : 1;
+    const int m = count > 0 ? cur.outs : 1;
     for (int j = tid; j < m; j += kAmpThreads) ends[(size_t)half * max_chi + j] = vs[j];
   }
 }
@@ -157,7 +174,7 @@ __global__ void __launch_bounds__(kAmpThreads) k_amp_dot(const double2* __restri
 }  // namespace
 
 // CTAs per half: about 1024 complex products per CTA and site, whose FP64
-// arithmetic then takes less time than the exchange
+// arithmetic then takes about the time of the exchange
 int amp_ctas(int max_chi, int n_sm) {
   const long long e = (long long)max_chi * max_chi;
   return (int)std::max<long long>(1, std::min<long long>(n_sm / 2, e / 1024));

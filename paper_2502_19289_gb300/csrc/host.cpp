@@ -1626,12 +1626,9 @@ static int level_sketch(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
 }
 
 // Full splits take the direct solver; the Jacobi solver keeps sketched splits,
-// runs with a sweep cap too low for it to be of use (a caller that lowers the
-// cap wants the error of a solve that does not converge), and the policy that
-// forces every product onto the tensor cores.
-// 12 sweeps are what the Jacobi first pass takes at most on the widths it is
-// used for; 4096 is the widest split of the ABI.
-constexpr int kDirectMinCap = 12, kDirectMaxWidth = 4096;
+// runs with a low sweep cap (kDirectMinCap), and the policy that forces every
+// product onto the tensor cores.  4096 is the widest split of the ABI.
+constexpr int kDirectMaxWidth = 4096;
 static bool use_direct(int n) {
   return g_max_sweeps >= kDirectMinCap && g_tc_mode != 2 && n <= kDirectMaxWidth;
 }

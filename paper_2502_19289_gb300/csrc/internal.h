@@ -296,7 +296,11 @@ void set_last_error(const std::string& msg);
 // FP32 FMA throughput probe: blocks x 256 threads x 8 chains x iters FMAs
 cudaError_t launch_fma_peak(float* out, int blocks, int iters, cudaStream_t s);
 
-// sweep cap of the Jacobi eigen-solves (ctebd_set_max_sweeps; default 30)
+// sweep cap of the Jacobi eigen-solves (ctebd_set_max_sweeps)
 int max_jacobi_sweeps();
+// Full splits take the direct solver unless the cap is below what the Jacobi
+// first pass takes at most on the widths it is used for: a caller that lowers
+// the cap that far wants the error of a solve that does not converge.
+constexpr int kDirectMinCap = 12;
 
 }  // namespace ctebd

@@ -101,13 +101,13 @@ struct NaDesc {
 };
 
 static int na_gemm(NaDesc& d, const GemmProb& p) {
-  const GemmProb* dp;
-  const long long off[2] = {0, gemm_tiles(p, false)};
-  const long long* doff;
-  int rc = d.put(&p, 1, &dp);
-  if (!rc) rc = d.put(off, 2, &doff);
-  if (rc) return rc;
-  NA_CUDA(launch_gemm<float>(dp, doff, 1, off[1], d.s));
+  struct One {
+    GemmProb p;
+    long long off[2];
+  } h = {p, {0, gemm_tiles(p, false)}};
+  const One* dp;
+  if (int rc = d.put(&h, 1, &dp)) return rc;
+  NA_CUDA(launch_gemm<float>(&dp->p, dp->off, 1, h.off[1], d.s));
   return CTEBD_OK;
 }
 
@@ -157,6 +157,34 @@ static int na_eig(NaDesc& d, unsigned char* S, void* acc, int npad, double floor
   return CTEBD_OK;
 }
 
+// Right singular vectors of diag(lam) Mbar by the direct solver (the handle
+// path's), in V: reflectors in the Gram area, eigenvectors in the refinement
+// accumulator, everything else in the area of the projection that follows.
+static int na_direct(NaDesc& d, unsigned char* S, int m, int n, int npad, const double* lamL, int* flag) {
+  int dev = 0, n_sm = 0;
+  NA_CUDA(cudaGetDevice(&dev));
+  NA_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  const size_t xchg = al256(dir_xchg_bytes<float>(m, n, 1, n_sm));
+  if (xchg + dir_scratch_doubles(n) * sizeof(double) > NA_OFF_G - NA_OFF_RFULL)
+    return na_fail(CTEBD_ERR_ARG, "split2_noalloc: internal: direct solver scratch");
+  DirProb q{};
+  q.M = S + NA_OFF_MBAR; q.lam = lamL; q.m = m; q.n = n; q.shift = 1; q.depth = dir_depth(n);
+  q.VR = S + NA_OFF_G;
+  q.Q0 = S + NA_OFF_W;
+  q.Q1 = reinterpret_cast<float*>(S + NA_OFF_W) + (size_t)n * n;
+  q.S = S + NA_OFF_V;
+  q.V = S + NA_OFF_V; q.ldv = npad; q.xld = n;
+  dir_carve(q, reinterpret_cast<double*>(S + NA_OFF_RFULL + xchg));
+  const DirProb* dq;
+  if (int rc = d.put(&q, 1, &dq)) return rc;
+  NA_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), d.s));
+  int launches = 0;
+  NA_CUDA(launch_dir_bidiag<float>(dq, 1, m, n, S + NA_OFF_RFULL, flag, n_sm, d.s));
+  NA_CUDA(launch_dir_tridiag<float>(dq, 1, n, &launches, d.s));
+  NA_CUDA(launch_dir_back<float>(dq, 1, n, d.s));
+  return CTEBD_OK;
+}
+
 // Rfull = Mbar V and its weighted column norms rho (the select follows)
 static int na_project(NaDesc& d, unsigned char* S, const void* V, int m, int n, int npad,
                       const double* lamL) {
@@ -170,18 +198,18 @@ static int na_project(NaDesc& d, unsigned char* S, const void* V, int m, int n, 
   // then rho_i / |v_i|^2 as the handle path does
   double* rho = (double*)(S + NA_OFF_RHO);
   NA_CUDA(cudaMemsetAsync(rho, 0, sizeof(double) * 2 * NA_N, d.s));
-  const void* R[2] = {S + NA_OFF_RFULL, V};
-  const int ms[2] = {m, n}, ns[2] = {n, n}, shs[2] = {1, 0}, lds[2] = {n, npad};
-  const double* lams[2] = {lamL, nullptr};
-  double* rhos[2] = {rho, rho + NA_N};
-  const void* const* dR; const int *dm, *dn, *dsh, *dld; const double* const* dL; double* const* drho;
-  if (int rc = d.put(R, 2, (const void* const**)&dR)) return rc;
-  if (int rc = d.put(ms, 2, &dm)) return rc;
-  if (int rc = d.put(ns, 2, &dn)) return rc;
-  if (int rc = d.put(shs, 2, &dsh)) return rc;
-  if (int rc = d.put(lds, 2, &dld)) return rc;
-  if (int rc = d.put(lams, 2, (const double* const**)&dL)) return rc;
-  if (int rc = d.put(rhos, 2, (double* const**)&drho)) return rc;
+  struct Cols {                  // one copy for all of the launch's descriptors
+    const void* R[2];
+    const double* lam[2];
+    double* rho[2];
+    int m[2], n[2], sh[2], ld[2];
+  } h = {{S + NA_OFF_RFULL, V}, {lamL, nullptr}, {rho, rho + NA_N}, {m, n}, {n, n}, {1, 0}, {n, npad}};
+  const Cols* dc;
+  if (int rc = d.put(&h, 1, &dc)) return rc;
+  const void* const* dR = dc->R;
+  const double* const* dL = dc->lam;
+  double* const* drho = dc->rho;
+  const int *dm = dc->m, *dn = dc->n, *dsh = dc->sh, *dld = dc->ld;
   NA_CUDA(launch_colnorm_batch<float>(dR, dm, dn, dld, dL, dsh, drho, 2, n, std::max(m, n), d.s));
   NA_CUDA(launch_rho_normalize(drho, drho + 1, dn, 1, n, d.s));
   return CTEBD_OK;
@@ -209,9 +237,14 @@ extern "C" int split2_noalloc(const void* theta, const double* lam_l, int chi_l,
   NaDesc d{S + NA_OFF_DESC, 0, s};
   // Mbar: copy of theta viewed (chi_l * 2) x (2 * chi_r)
   NA_CUDA(cudaMemcpyAsync(S + NA_OFF_MBAR, theta, (size_t)m * n * NA_CPLX, cudaMemcpyDeviceToDevice, s));
-  // pass 1: Gram of Mbar weighted by lambda_l^2 (row a of theta carries lambda_l[a])
-  NA_CUDA(cudaMemsetAsync(S + NA_OFF_G, 0, (size_t)npad * npad * NA_CPLX, s));
-  {
+  void* V = S + NA_OFF_V;
+  const bool direct = max_jacobi_sweeps() >= kDirectMinCap;
+  int* flag = (int*)(S + NA_OFF_CNT);   // a bounded wait of the direct solver ran out
+  if (direct) {
+    if (int rc = na_direct(d, S, m, n, npad, lam_l, flag)) return rc;
+  } else {
+    // pass 1: Gram of Mbar weighted by lambda_l^2 (row a of theta carries lambda_l[a])
+    NA_CUDA(cudaMemsetAsync(S + NA_OFF_G, 0, (size_t)npad * npad * NA_CPLX, s));
     GemmProb p{};
     p.M = n; p.N = n; p.K = m; p.batch = 1;
     p.A = S + NA_OFF_MBAR; p.lda = n; p.opA = 1;
@@ -219,10 +252,10 @@ extern "C" int split2_noalloc(const void* theta, const double* lam_l, int chi_l,
     p.C = S + NA_OFF_G; p.ldc = npad;
     p.kw = lam_l; p.kw_shift = 1; p.alpha = 1.0;
     if (int rc = na_gemm(d, p)) return rc;
+    if (int rc = na_eig(d, S, V, npad, 1.0, 4.0, 0.0, 0.0)) return rc;
   }
-  void* V = S + NA_OFF_V;
-  if (int rc = na_eig(d, S, V, npad, 1.0, 4.0, 0.0, 0.0)) return rc;
   double res[8];
+  int timed_out = 0;
   auto select = [&](const void* Vc) -> int {
     if (int rc = na_project(d, S, Vc, m, n, npad, lam_l)) return rc;
     SelProb sp{};
@@ -235,15 +268,17 @@ extern "C" int split2_noalloc(const void* theta, const double* lam_l, int chi_l,
     const double eps32 = 1.1920928955078125e-07;
     NA_CUDA(launch_select(dsp, 1, chi_max, cutoff, 16.0 * eps32, 1024.0 * eps32, 1e-12, s));
     NA_CUDA(cudaMemcpyAsync(res, S + NA_OFF_RES, sizeof(res), cudaMemcpyDeviceToHost, s));
+    if (direct) NA_CUDA(cudaMemcpyAsync(&timed_out, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
     d.off = 0;
+    if (timed_out) return na_fail(CTEBD_ERR_TIMEOUT, "split2_noalloc: a wait of the direct solver timed out");
     return CTEBD_OK;
   };
   if (int rc = select(V)) return rc;
-  // pass 2 wherever something is discarded, or a cutoff is set and pass 1 left
+  // Jacobi: pass 2 wherever something is discarded, or a cutoff is set and pass 1 left
   // unresolved directions (relative thresholds and the moved-weight stopping
   // rule of the handle path)
-  if ((int)res[0] < n || (cutoff > 0 && (int)res[6] < n)) {
+  if (!direct && ((int)res[0] < n || (cutoff > 0 && (int)res[6] < n))) {
     NA_CUDA(cudaMemsetAsync(S + NA_OFF_G, 0, (size_t)npad * npad * NA_CPLX, s));
     GemmProb p{};
     p.M = n; p.N = n; p.K = m; p.batch = 1;
