@@ -383,12 +383,12 @@ struct Work {
 enum KernelKind {
   KK_GEMM_MERGE, KK_GEMM_U, KK_GEMM_GRAM, KK_GEMM_PROJ, KK_EIG_INIT, KK_EIG_INNER, KK_EIG_APPLY,
   KK_COLNORM, KK_SELECT, KK_GATHER, KK_ONEQ, KK_AMP, KK_GEMM_SKETCH, KK_CHOL, KK_MLP,
-  KK_BIDIAG, KK_TRIDIAG, KK_BACK, KK_COUNT
+  KK_BIDIAG, KK_TRIDIAG, KK_BACK, KK_SMALL, KK_COUNT
 };
 static const char* kKindNames[KK_COUNT] = {
   "gemm_merge", "gemm_apply_u", "gemm_gram", "gemm_project", "eig_init", "eig_inner", "eig_apply",
   "colnorm", "select", "gather", "apply_1q", "amplitude", "gemm_sketch", "cholqr", "mlp_forward",
-  "bidiag", "tridiag_eig", "back_transform"};
+  "bidiag", "tridiag_eig", "back_transform", "small_chain"};
 
 struct Prof {
   bool on = false;
@@ -473,6 +473,9 @@ struct ctebd_mps {
   unsigned char* dir_scr = nullptr;    // direct solver: exchange buffers, per-problem scratch (high-water)
   size_t dir_cap = 0;                  // in bytes
   int n_sm = 0;
+  double* small_res = nullptr;         // results of k_small_chain (high-water), and the pinned copy
+  double* h_small = nullptr;
+  size_t small_cap = 0;                // in doubles
   cudaStream_t side = nullptr;     // second branch of the device-side sweep graphs
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   void* arena = nullptr;
@@ -578,6 +581,8 @@ extern "C" int mps_destroy(ctebd_mps* m) {
   if (m->eig_scr) cudaFree(m->eig_scr);
   if (m->pack_scr) cudaFree(m->pack_scr);
   if (m->dir_scr) cudaFree(m->dir_scr);
+  if (m->small_res) cudaFree(m->small_res);
+  if (m->h_small) cudaFreeHost(m->h_small);
   if (m->h_res) cudaFreeHost(m->h_res);
   m->stage.release();
   m->prof.release();
@@ -1765,6 +1770,106 @@ static int level_solve(ctebd_mps* m, std::vector<Work>& ws, Level& L, const std:
   return level_project_select(m, ws, L, ref);
 }
 
+// One split's results: the numbers of the split log, and its place in it
+// (level by level, clusters in order).
+struct SplitRow {
+  int lev, i;
+  double row[14];
+};
+
+// Whether one CTA can do all splits of a cluster.
+// The rank at bond q0 + j is at most min(chi_max, chi_L 2^j, chi_R 2^(k - j)).
+static int rank_bound(const ctebd_mps* m, const Work& w, int j) {
+  return (int)std::min({(long long)m->cfg.chi_max, (long long)w.chiL << j, (long long)w.chiR << (w.k - j)});
+}
+static bool use_small(const ctebd_mps* m, const Work& w, size_t& smem) {
+  if (!use_direct(1) || w.k > 12) return false;   // SmallProb holds 12 sites
+  if (m->cfg.sketch_oversample > 0 && !m->fp64)
+    for (int j = 0; j < w.k - 1; j++)
+      if (w.hint[j] > 0) return false;          // a sketched split was asked for
+  smem = 0;
+  for (int j = w.k - 1; j >= 1; j--) {
+    const int mm = w.chiL << j, nn = 2 * (j + 1 < w.k ? rank_bound(m, w, j + 1) : w.chiR);
+    if (!small_fits(mm, nn)) return false;
+    smem = std::max(smem, small_smem(mm, nn));
+  }
+  return true;
+}
+
+// All splits of the clusters `sel` (indices into ws) in one launch; the results
+// are read by small_finish, after other work has been queued.
+static int small_start(ctebd_mps* m, std::vector<Work>& ws, const std::vector<int>& sel, size_t smem) {
+  std::vector<SmallProb> sp(sel.size());
+  size_t rows = 0;
+  double fl = 0;
+  for (int i : sel) rows += ws[i].k - 1;
+  if (8 * rows > m->small_cap) {   // device results and their pinned copy
+    CUDA_TRY(cudaStreamSynchronize(m->stream));
+    if (m->small_res) CUDA_TRY(cudaFree(m->small_res));
+    if (m->h_small) CUDA_TRY(cudaFreeHost(m->h_small));
+    m->small_res = m->h_small = nullptr;
+    m->small_cap = 0;
+    const size_t want = 8 * (rows + rows / 2 + 64);
+    if (cudaMalloc(&m->small_res, want * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost(&m->h_small, want * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(CTEBD_ERR_OOM, "split results");
+    }
+    m->small_cap = want;
+  }
+  double* res = m->small_res;
+  for (size_t a = 0; a < sel.size(); a++) {
+    Work& w = ws[sel[a]];
+    SmallProb& p = sp[a];
+    p.theta = w.bufA; p.rem = w.bufB; p.lam = m->lam[w.q0];
+    p.chiL = w.chiL; p.chiR = w.chiR; p.k = w.k;
+    p.res = res;
+    res += 8 * (w.k - 1);
+    for (int j = 0; j < w.k; j++) {
+      const size_t right = j + 1 < w.k ? rank_bound(m, w, j + 1) : w.chiR, left = j > 0 ? rank_bound(m, w, j) : w.chiL;
+      TRY(ensure_site(m, w.q0 + j, left * 2 * right));
+      p.site[j] = m->site[w.q0 + j];
+      p.lam_out[j] = m->lam[w.q0 + j];
+      if (j > 0) {
+        const double mm = (double)(w.chiL << j), nn = 2.0 * right;
+        fl += 16.0 * mm * nn * std::min(mm, nn);
+      }
+    }
+  }
+  const SmallProb* dp;
+  TRY(m->stage.push(sp.data(), sp.size(), &dp));
+  ProfScope ps(m->prof, m->stream, KK_SMALL, fl, 0);
+  const double floor_rel = m->fp64 ? 1e-13 : 1e-6;
+  CUDA_TRY(m->fp64 ? launch_small_chain<double>(dp, (int)sp.size(), smem, m->cfg.chi_max, m->cfg.cutoff,
+                                                floor_rel * floor_rel, g_max_sweeps, m->stream)
+                   : launch_small_chain<float>(dp, (int)sp.size(), smem, m->cfg.chi_max, m->cfg.cutoff,
+                                               floor_rel * floor_rel, g_max_sweeps, m->stream));
+  CUDA_TRY(cudaMemcpyAsync(m->h_small, m->small_res, sizeof(double) * 8 * rows, cudaMemcpyDeviceToHost, m->stream));
+  return CTEBD_OK;
+}
+
+static int small_finish(ctebd_mps* m, std::vector<Work>& ws, const std::vector<int>& sel, std::vector<SplitRow>& rows) {
+  CUDA_TRY(cudaStreamSynchronize(m->stream));
+  const double* res = m->h_small;
+  for (int i : sel) {
+    Work& w = ws[i];
+    for (int lev = 1; lev < w.k; lev++, res += 8) {
+      const int j = w.k - lev, bnd = w.q0 + j, n = 2 * w.rdim, mm = w.chiL << j, r = (int)res[0];
+      if (res[5] != 0)
+        return fail(CTEBD_ERR_NUMERIC, "one-sided Jacobi: a split is still rotating after " +
+                                           std::to_string(g_max_sweeps) + " sweeps");
+      if (!(res[3] > 0) || !std::isfinite(res[2])) return fail(CTEBD_ERR_NUMERIC, "split: non-finite or zero weight");
+      if (r < 1 || r > n || r > m->cfg.chi_max)
+        return fail(CTEBD_ERR_NUMERIC, "split: rank out of range (" + std::to_string(r) + ")");
+      m->chi[bnd] = r;
+      w.rdim = r;
+      rows.push_back({lev, i, {(double)w.q0, (double)w.k, (double)bnd, (double)mm, (double)n, (double)r, res[1], res[2],
+                               0.0, (double)n, res[4], (double)w.hint[j - 1], 0.0, 0.0}});
+    }
+  }
+  return CTEBD_OK;
+}
+
 // k-1 splits, right to left (Fig. 2 with the truncation of Fig. 3)
 static int split_levels(ctebd_mps* m, std::vector<Work>& ws, std::vector<std::vector<double>>& fs,
                         uint64_t step_key) {
@@ -1772,11 +1877,24 @@ static int split_levels(ctebd_mps* m, std::vector<Work>& ws, std::vector<std::ve
   const int JB = eig_block(f64);
   const int p_over = m->cfg.sketch_oversample;
   fs.assign(ws.size(), {});
+  std::vector<SplitRow> rows;
+  // narrow clusters: all their splits in one launch
+  std::vector<int> small;
+  std::vector<char> is_small(ws.size(), 0);
+  size_t smem = 0;
+  for (size_t i = 0; i < ws.size(); i++) {
+    size_t s1;
+    if (!use_small(m, ws[i], s1)) continue;
+    small.push_back((int)i);
+    is_small[i] = 1;
+    smem = std::max(smem, s1);
+  }
+  if (!small.empty()) TRY(small_start(m, ws, small, smem));
   int kmax = 0;
-  for (auto& w : ws) kmax = std::max(kmax, w.k);
+  for (size_t i = 0; i < ws.size(); i++) if (!is_small[i]) kmax = std::max(kmax, ws[i].k);
   for (int lev = 1; lev < kmax; lev++) {
     Level L;
-    for (size_t i = 0; i < ws.size(); i++) if (ws[i].k - 1 >= lev) L.act.push_back((int)i);
+    for (size_t i = 0; i < ws.size(); i++) if (!is_small[i] && ws[i].k - 1 >= lev) L.act.push_back((int)i);
     if (L.act.empty()) break;
     const int na = (int)L.act.size();
     for (auto* v : {&L.mm, &L.nn, &L.npad, &L.shift, &L.ne, &L.nepad, &L.nbv, &L.vld}) v->resize(na);
@@ -1866,13 +1984,9 @@ static int split_levels(ctebd_mps* m, std::vector<Work>& ws, std::vector<std::ve
       maxe = std::max(maxe, std::max((long long)r * L.nn[a], (long long)r * L.mm[a]));
       m->chi[bnd] = r;
       w.rdim = r;
-      m->logF += std::log(f);
-      fs[L.act[a]].push_back(f);
-      const double row[8] = {(double)w.q0, (double)w.k, (double)bnd, (double)L.mm[a], (double)L.nn[a], (double)r, f, W};
-      m->splitlog.insert(m->splitlog.end(), row, row + 8);
-      const double extra[6] = {(double)L.sk[a], (double)L.ne[a], res[4], (double)w.hint[j - 1],
-                               (double)L.sw1[a], (double)L.sw2[a]};
-      m->splitlog2.insert(m->splitlog2.end(), extra, extra + 6);
+      rows.push_back({lev, L.act[a], {(double)w.q0, (double)w.k, (double)bnd, (double)L.mm[a], (double)L.nn[a], (double)r,
+                                      f, W, (double)L.sk[a], (double)L.ne[a], res[4], (double)w.hint[j - 1],
+                                      (double)L.sw1[a], (double)L.sw2[a]}});
     }
     const GatherProb* dgp;
     TRY(m->stage.push(gp.data(), gp.size(), &dgp));
@@ -1882,8 +1996,20 @@ static int split_levels(ctebd_mps* m, std::vector<Work>& ws, std::vector<std::ve
     CUDA_TRY(f64 ? launch_gather<double>(dgp, (int)gp.size(), maxe, m->stream)
                  : launch_gather<float>(dgp, (int)gp.size(), maxe, m->stream));
   }
-  // leftmost site of every cluster: the remainder (chiL*2 x r1)
-  for (auto& w : ws) {
+  if (!small.empty()) TRY(small_finish(m, ws, small, rows));
+  std::sort(rows.begin(), rows.end(), [](const SplitRow& a, const SplitRow& b) {
+    return a.lev != b.lev ? a.lev < b.lev : a.i < b.i;
+  });
+  for (const SplitRow& r : rows) {
+    m->logF += std::log(r.row[6]);
+    fs[r.i].push_back(r.row[6]);
+    m->splitlog.insert(m->splitlog.end(), r.row, r.row + 8);
+    m->splitlog2.insert(m->splitlog2.end(), r.row + 8, r.row + 14);
+  }
+  // leftmost site of every other cluster: the remainder (chiL*2 x r1)
+  for (size_t i = 0; i < ws.size(); i++) {
+    Work& w = ws[i];
+    if (is_small[i]) continue;
     const size_t elems = (size_t)w.chiL * 2 * w.rdim;
     TRY(ensure_site(m, w.q0, elems));
     CUDA_TRY(cudaMemcpyAsync(m->site[w.q0], w.bufA, elems * m->esz, cudaMemcpyDeviceToDevice, m->stream));

@@ -97,6 +97,22 @@ cudaError_t launch_dir_tridiag(const DirProb* probs, int count, int max_n, int* 
 template <typename R>
 cudaError_t launch_dir_back(const DirProb* probs, int count, int max_n, cudaStream_t s);
 
+// A cluster whose k - 1 splits run in one CTA (small_split.cu).
+struct SmallProb {
+  const void* theta;      // chi_L x 2^k x chi_R
+  void* rem;              // remainder between levels (at least theta's size)
+  const double* lam;      // left spectrum
+  int chiL, chiR, k;
+  void* site[12];         // [j]: site q0 + j (capacity for the largest possible ranks)
+  double* lam_out[12];    // [j], j >= 1: spectrum of bond q0 + j
+  double* res;            // 8 per level: r, f, W, kept, rank before the chi_max cap, 1 if not converged
+};
+bool small_fits(int m, int n);       // rows and columns of the first split
+size_t small_smem(int m, int n);
+template <typename R>
+cudaError_t launch_small_chain(const SmallProb* d_probs, int count, size_t smem, int chi_max, double cutoff,
+                               double floor2, int max_sweeps, cudaStream_t s);
+
 // Per-problem truncation inputs/outputs of one split level.
 struct SelProb {
   const double* rho;   // n weighted column norms
