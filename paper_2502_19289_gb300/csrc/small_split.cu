@@ -85,13 +85,15 @@ __global__ void __launch_bounds__(kSmThreads, 1)
   // Vectors far below the largest one are what rounding left of a rank-deficient matrix.  They are not rotated
   // (kQuiet, of the squared norm), and all below the truncation's numerical-zero floor are dropped: the weights of
   // their directions, taken from Z, would be their overlap with the large ones.
-  // Couplings (squared, relative) up to kSkip are left: far below the tensors' rounding, or in FP64 ten times the
-  // rotations' own rounding.  A sweep with a rotation by more than sqrt(kAgain), or at a coupling above it, is
-  // followed by another; what is left after one without is far smaller (of second order, and 1e-7 of it, the
-  // angles' rounding).  The angle counts as well as the coupling: between equal norms a tiny coupling turns the two
-  // by 45 degrees, and with them their couplings to others, from pairs still to come to pairs already done.
+  // Couplings (squared, relative) up to kLow are left: far below the tensors' rounding, or in FP64 at the level of
+  // the sums' own; up to kSkip, ten times the rotations' rounding, only small turns are made (between equal norms
+  // noise would turn by 45 degrees for ever).  A sweep with a rotation by more than sqrt(kAgain), or at a coupling
+  // above it, is followed by another; what is left after one without is far smaller (of second order, and 1e-7 of
+  // it, the angles' rounding).  The angle counts as well as the coupling: between equal norms a tiny coupling turns
+  // the two by 45 degrees, and with them their couplings to others, from pairs still to come to pairs already done.
   constexpr double kTiny = 1e-290;
-  constexpr float kQuiet = 1e-29f, kSkip = sizeof(S) == 4 ? 1e-20f : 3.2e-30f, kAgain = sizeof(S) == 4 ? 1e-10f : 1e-18f;
+  constexpr float kQuiet = 1e-29f, kLow = sizeof(S) == 4 ? 1e-20f : 3e-31f, kSkip = sizeof(S) == 4 ? 1e-20f : 3.2e-30f;
+  constexpr float kAgain = sizeof(S) == 4 ? 1e-10f : 1e-18f;
   const CS* src = reinterpret_cast<const CS*>(P.theta);
   int rdim = P.chiR;
   for (int lev = 1; lev < P.k; lev++) {
@@ -184,20 +186,21 @@ __global__ void __launch_bounds__(kSmThreads, 1)
           const float rf = big ? rsqrtf(af) * rsqrtf(df) : 0.f;
           const float gx = (float)(g.x * (double)rf), gy = (float)(g.y * (double)rf);
           const float g2 = fmaf(gx, gx, gy * gy);
-          if (g2 > kSkip) {
+          if (g2 > kLow) {
             const float ig = rsqrtf(g2), zeta = (float)(d - a) * 0.5f * rf * ig, az = fabsf(zeta);
             const float tt = az < 1e9f ? 1.f / (az + sqrtf(fmaf(az, az, 1.f))) : 0.5f / az, st = (zeta >= 0.f ? tt : -tt) * ig;
+            const bool turn = g2 > kSkip || tt * tt < 1e-6f;
             const double tx = (double)(st * gx), ty = -(double)(st * gy);
             const double n2 = fma(tx, tx, fma(ty, ty, 1.0));
             double co = (double)rsqrtf((float)n2);
             co = fma(co, fma(-0.5 * n2 * co, co, 0.5), co);
             co = fma(co, fma(-0.5 * n2 * co, co, 0.5), co);
             const double sx = co * tx, sy = co * ty;
-            if (have) {    // u' = co u - s v, v' = co v + conj(s) u
+            if (have && turn) {    // u' = co u - s v, v' = co v + conj(s) u
               X[p * ldx + c0] = make_double2(fma(co, u.x, fma(-sx, v.x, sy * v.y)), fma(co, u.y, fma(-sx, v.y, -sy * v.x)));
               X[q * ldx + c0] = make_double2(fma(co, v.x, fma(sx, u.x, sy * u.y)), fma(co, v.y, fma(sx, u.y, -sy * u.x)));
             }
-            if (c0 == 0 && fmaxf(g2, tt * tt) > kAgain) sig = 1;
+            if (c0 == 0 && turn && fmaxf(g2, tt * tt) > kAgain) sig = 1;
           }
           __syncwarp();
         }
