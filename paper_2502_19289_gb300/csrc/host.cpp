@@ -306,40 +306,111 @@ extern "C" int cluster_unitary(const ctebd_gate* gates, int n_gates, const ctebd
 }
 
 // ---------------------------------------------------------------------------
-// Device staging of small descriptor arrays (pinned host -> device, bump)
+// Staging: pinned host memory, and device memory of the same size behind it.
+// Descriptor arrays are copied through both (push), other data through the
+// host side only (copy_to, and reads).  A page-locked block costs 0.11 ms to
+// make and 0.17 ms to free whatever its size up to 2 MB (8 MB: 0.22 / 0.25),
+// so the handle's one first block holds its other pinned words too; larger
+// blocks are made when a call needs them.
 // ---------------------------------------------------------------------------
 struct Staging {
+  static constexpr size_t kFirst = (size_t)1 << 20, kMax = (size_t)8 << 20;
   unsigned char* h = nullptr;
   unsigned char* d = nullptr;
   size_t cap = 0, off = 0;
   cudaStream_t s = nullptr;
-  int init(size_t c, cudaStream_t st) {
+  std::vector<std::pair<unsigned char*, unsigned char*>> full;   // outgrown blocks, in use until reset
+  unsigned char *first_h = nullptr, *first_d = nullptr;
+  // the first block, with extra_h / extra_d bytes behind it for the caller
+  int init(cudaStream_t st, size_t extra_h, size_t extra_d) {
     s = st;
-    cap = c;
-    CUDA_TRY(cudaMallocHost(&h, cap));
-    CUDA_TRY(cudaMalloc(&d, cap));
+    CUDA_TRY(cudaMallocHost(&first_h, kFirst + extra_h));
+    CUDA_TRY(cudaMalloc(&first_d, kFirst + extra_d));
+    h = first_h;
+    d = first_d;
+    cap = kFirst;
     return CTEBD_OK;
   }
+  void drop_full() {
+    for (auto& b : full) {
+      if (b.first != first_h) cudaFreeHost(b.first);
+      if (b.second != first_d) cudaFree(b.second);
+    }
+    full.clear();
+  }
   void release() {
-    if (h) cudaFreeHost(h);
-    if (d) cudaFree(d);
-    h = d = nullptr;
+    drop_full();
+    if (h && h != first_h) cudaFreeHost(h);
+    if (d && d != first_d) cudaFree(d);
+    if (first_h) cudaFreeHost(first_h);
+    if (first_d) cudaFree(first_d);
+    h = d = first_h = first_d = nullptr;
   }
   // Callers reset only after a stream synchronisation.
-  void reset() { off = 0; }
-  template <typename T>
-  int push(const T* src, size_t count, const T** out) {
-    const size_t bytes = sizeof(T) * std::max<size_t>(count, 1);
+  void reset() {
+    off = 0;
+    if (!full.empty()) drop_full();
+  }
+  // room for `bytes` at h + *at and d + *at
+  int room(size_t bytes, size_t* at) {
     const size_t need = (bytes + 255) & ~size_t(255);
     if (off + need > cap) {
-      CUDA_TRY(cudaStreamSynchronize(s));
+      if (need > kMax) {
+        CUDA_TRY(cudaStreamSynchronize(s));
+        return fail(CTEBD_ERR_OOM, "staging buffer too small");
+      }
+      if (cap < kMax) {
+        size_t want = 4 * cap;
+        while (want < need) want *= 2;
+        want = std::min(want, kMax);
+        unsigned char *nh = nullptr, *nd = nullptr;
+        CUDA_TRY(cudaMallocHost(&nh, want));
+        if (cudaMalloc(&nd, want) != cudaSuccess) {
+          cudaGetLastError();
+          cudaFreeHost(nh);
+          return fail(CTEBD_ERR_OOM, "staging buffer");
+        }
+        full.push_back({h, d});
+        h = nh;
+        d = nd;
+        cap = want;
+      } else {
+        CUDA_TRY(cudaStreamSynchronize(s));
+      }
       off = 0;
-      if (need > cap) return fail(CTEBD_ERR_OOM, "staging buffer too small");
     }
-    std::memcpy(h + off, src, sizeof(T) * count);
-    CUDA_TRY(cudaMemcpyAsync(d + off, h + off, sizeof(T) * count, cudaMemcpyHostToDevice, s));
-    *out = reinterpret_cast<const T*>(d + off);
+    *at = off;
     off += need;
+    return CTEBD_OK;
+  }
+  template <typename T>
+  int push(const T* src, size_t count, const T** out) {
+    size_t at;
+    TRY(room(sizeof(T) * std::max<size_t>(count, 1), &at));
+    std::memcpy(h + at, src, sizeof(T) * count);
+    CUDA_TRY(cudaMemcpyAsync(d + at, h + at, sizeof(T) * count, cudaMemcpyHostToDevice, s));
+    *out = reinterpret_cast<const T*>(d + at);
+    return CTEBD_OK;
+  }
+  // several arrays in one copy: add() each, then push_all(); ptr() after it
+  struct Set {
+    std::vector<unsigned char> bytes;
+    const unsigned char* base = nullptr;
+    template <typename T> size_t add(const T* src, size_t count) {
+      const size_t at = (bytes.size() + 15) & ~size_t(15);
+      bytes.resize(at + sizeof(T) * std::max<size_t>(count, 1));
+      std::memcpy(bytes.data() + at, src, sizeof(T) * count);
+      return at;
+    }
+    template <typename T> const T* ptr(size_t at) const { return reinterpret_cast<const T*>(base + at); }
+  };
+  int push_all(Set& set) { return push(set.bytes.data(), set.bytes.size(), &set.base); }
+  // host data to a device buffer of its own
+  int copy_to(void* dst, const void* src, size_t bytes) {
+    size_t at;
+    TRY(room(bytes, &at));
+    std::memcpy(h + at, src, bytes);
+    CUDA_TRY(cudaMemcpyAsync(dst, h + at, bytes, cudaMemcpyHostToDevice, s));
     return CTEBD_OK;
   }
 };
@@ -454,8 +525,11 @@ struct ctebd_mps {
   std::vector<int> chi;
   std::vector<void*> site;
   std::vector<size_t> site_cap;
+  unsigned char* site_block = nullptr;   // the initial product state's sites
   std::vector<double*> lam;
   int lam_cap = 0;
+  double* lam_block = nullptr;     // all bonds' spectra, in one allocation
+  cudaMemPool_t pool = nullptr;    // sites and other stream-ordered allocations
   double logF = 0;
   std::vector<double> splitlog;
   std::vector<double> splitlog2;   // per split: sketched, eigen-dim, rank before cap, hint,
@@ -473,25 +547,39 @@ struct ctebd_mps {
   unsigned char* dir_scr = nullptr;    // direct solver: exchange buffers, per-problem scratch (high-water)
   size_t dir_cap = 0;                  // in bytes
   int n_sm = 0;
-  double* small_res = nullptr;         // results of k_small_chain (high-water), and the pinned copy
+  double* small_res = nullptr;         // results of k_small_chain and the pinned copy, behind the staging block
   double* h_small = nullptr;
-  size_t small_cap = 0;                // in doubles
   cudaStream_t side = nullptr;     // second branch of the device-side sweep graphs
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   void* arena = nullptr;
   size_t arena_cap = 0;
   Staging stage;
-  double* h_res = nullptr;       // pinned results of select (8 per problem)
-  size_t h_res_cap = 0;
+  double* h_res = nullptr;       // pinned results of select: 16 doubles per problem, then the kernels' wait flag
+  double* h_raw = nullptr;       // as they arrive, by work item
+  size_t h_res_cap = 0;          // in problems
   std::map<int, Work> pending;
   Prof prof;
 };
 
+// Stream-ordered memory from the handle's pool, which keeps up to kPoolKeep
+// bytes between calls: the device's default pool gives everything back at each
+// synchronisation (95 us for an allocation and its release).
+constexpr uint64_t kPoolKeep = (uint64_t)1 << 30;
+template <typename T> static cudaError_t pool_alloc(ctebd_mps* m, T** p, size_t bytes) {
+  return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, m->pool, m->stream);
+}
+
+static bool in_site_block(const ctebd_mps* m, const void* p) {
+  const unsigned char* c = static_cast<const unsigned char*>(p);
+  return m->site_block && c >= m->site_block && c < m->site_block + 32 * (size_t)m->n;
+}
+
 static int ensure_site(ctebd_mps* m, int q, size_t elems) {
   if (m->site_cap[q] >= elems) return CTEBD_OK;
-  if (m->site[q]) CUDA_TRY(cudaFreeAsync(m->site[q], m->stream));
+  if (m->site[q] && !in_site_block(m, m->site[q])) CUDA_TRY(cudaFreeAsync(m->site[q], m->stream));
   m->site[q] = nullptr;
-  CUDA_TRY(cudaMallocAsync(&m->site[q], std::max<size_t>(elems, 1) * m->esz, m->stream));
+  m->site_cap[q] = 0;
+  CUDA_TRY(pool_alloc(m, &m->site[q], std::max<size_t>(elems, 1) * m->esz));
   m->site_cap[q] = elems;
   return CTEBD_OK;
 }
@@ -530,34 +618,58 @@ extern "C" int mps_create(const ctebd_config* cfg, void* cuda_stream, ctebd_mps*
   m->site_cap.assign(m->n, 0);
   m->lam_cap = cfg->chi_max;
   m->lam.assign(m->n + 1, nullptr);
-  int rc = m->stage.init(8 << 20, m->stream);
+  // a step has at most n / 2 clusters and fewer than n splits
+  m->h_res_cap = std::min(4096, std::max(m->n / 2, 1));
+  const size_t raw = 16 * (size_t)std::max(m->n / 2, 1), small = 8 * (size_t)m->n;
+  int rc = m->stage.init(m->stream, sizeof(double) * (16 * (m->h_res_cap + 1) + raw + small), sizeof(double) * small);
   if (rc) { mps_destroy(m); return rc; }
+  m->h_res = reinterpret_cast<double*>(m->stage.first_h + Staging::kFirst);
+  m->h_raw = m->h_res + 16 * (m->h_res_cap + 1);
+  m->h_small = m->h_raw + raw;
+  m->small_res = reinterpret_cast<double*>(m->stage.first_d + Staging::kFirst);
   int dev = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&m->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || m->n_sm < 1) {
     mps_destroy(m);
     return fail(CTEBD_ERR_CUDA, "mps_create: device attributes");
   }
-  // 16 doubles per problem, then the copy of the kernels' wait flag
-  if (cudaMallocHost(&m->h_res, 16 * sizeof(double) * (4096 + 1)) != cudaSuccess) { mps_destroy(m); return fail(CTEBD_ERR_OOM, "pinned"); }
-  m->h_res_cap = 4096;
-  std::vector<double> one(1, 1.0);
-  for (int b = 0; b <= m->n; b++) {
-    if (cudaMalloc(&m->lam[b], sizeof(double) * m->lam_cap) != cudaSuccess) { mps_destroy(m); return fail(CTEBD_ERR_OOM, "lambda"); }
-    cudaMemcpyAsync(m->lam[b], one.data(), sizeof(double), cudaMemcpyHostToDevice, m->stream);
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  uint64_t keep = kPoolKeep;
+  if (cudaMemPoolCreate(&m->pool, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(m->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    mps_destroy(m);
+    return fail(CTEBD_ERR_CUDA, "mps_create: memory pool");
   }
-  // |0> on every site: (1, 2, 1) tensor [1, 0]
-  std::vector<double> zero_state(4, 0.0);
-  zero_state[0] = 1.0;
+  // spectra [1]: one allocation, 256-byte rows
+  const size_t lam_ld = ((size_t)m->lam_cap + 31) / 32 * 32;
+  if (cudaMalloc(&m->lam_block, sizeof(double) * lam_ld * (m->n + 1)) != cudaSuccess) {
+    cudaGetLastError();
+    mps_destroy(m);
+    return fail(CTEBD_ERR_OOM, "lambda");
+  }
+  std::vector<double> one(m->n + 1, 1.0);
+  for (int b = 0; b <= m->n; b++) m->lam[b] = m->lam_block + lam_ld * b;
+  cudaMemcpy2DAsync(m->lam_block, sizeof(double) * lam_ld, one.data(), sizeof(double), sizeof(double), m->n + 1,
+                    cudaMemcpyHostToDevice, m->stream);
+  // |0> on every site: (1, 2, 1) tensor [1, 0], first in one block of 32-byte places
+  const size_t place = 32;
+  if (pool_alloc(m, &m->site_block, place * m->n) != cudaSuccess) {
+    cudaGetLastError();
+    mps_destroy(m);
+    return fail(CTEBD_ERR_OOM, "sites");
+  }
+  std::vector<unsigned char> zero_state(place * m->n, 0);
   for (int q = 0; q < m->n; q++) {
-    if (ensure_site(m, q, 2) != CTEBD_OK) { mps_destroy(m); return CTEBD_ERR_OOM; }
-    if (m->fp64) {
-      cudaMemcpyAsync(m->site[q], zero_state.data(), 32, cudaMemcpyHostToDevice, m->stream);
-    } else {
-      float z[4] = {1.f, 0.f, 0.f, 0.f};
-      cudaMemcpyAsync(m->site[q], z, 16, cudaMemcpyHostToDevice, m->stream);
-    }
+    unsigned char* z = zero_state.data() + place * q;
+    if (m->fp64) *reinterpret_cast<double*>(z) = 1.0;
+    else *reinterpret_cast<float*>(z) = 1.f;
+    m->site[q] = m->site_block + place * q;
+    m->site_cap[q] = 2;
   }
+  cudaMemcpyAsync(m->site_block, zero_state.data(), zero_state.size(), cudaMemcpyHostToDevice, m->stream);
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) { mps_destroy(m); return fail(CTEBD_ERR_CUDA, "mps_create: init"); }
   *out = m;
   return CTEBD_OK;
@@ -571,19 +683,19 @@ extern "C" int mps_destroy(ctebd_mps* m) {
   for (auto& kv : m->pending) {
     Work& w = kv.second;
     if (w.owned)
-      for (auto& pb : work_buffers(m, w)) if (*pb.first) cudaFree(*pb.first);
+      for (auto& pb : work_buffers(m, w)) if (*pb.first) cudaFreeAsync(*pb.first, m->stream);
   }
-  for (void* p : m->site) if (p) cudaFree(p);
-  for (double* p : m->lam) if (p) cudaFree(p);
+  for (void* p : m->site) if (p && !in_site_block(m, p)) cudaFreeAsync(p, m->stream);
+  if (m->site_block) cudaFreeAsync(m->site_block, m->stream);
+  if (m->stream) cudaStreamSynchronize(m->stream);
+  if (m->pool) cudaMemPoolDestroy(m->pool);
+  if (m->lam_block) cudaFree(m->lam_block);
   if (m->arena) cudaFree(m->arena);
   if (m->mlp) cudaFree(m->mlp);
   if (m->tc_err) cudaFree(m->tc_err);
   if (m->eig_scr) cudaFree(m->eig_scr);
   if (m->pack_scr) cudaFree(m->pack_scr);
   if (m->dir_scr) cudaFree(m->dir_scr);
-  if (m->small_res) cudaFree(m->small_res);
-  if (m->h_small) cudaFreeHost(m->h_small);
-  if (m->h_res) cudaFreeHost(m->h_res);
   m->stage.release();
   m->prof.release();
   if (m->side) cudaStreamDestroy(m->side);
@@ -694,11 +806,12 @@ static int launch_gemm_group(ctebd_mps* m, const std::vector<GemmProb>& probs, i
         poff[i + 1] = poff[i] + tc_packed_pack_blocks(q.g);
         toff[i + 1] = toff[i] + tc_packed_tiles(q.g);
       }
-      const PackedProb* dpp;
-      const long long *dpo, *dto;
-      TRY(m->stage.push(pp.data(), pp.size(), &dpp));
-      TRY(m->stage.push(poff.data(), poff.size(), &dpo));
-      TRY(m->stage.push(toff.data(), toff.size(), &dto));
+      Staging::Set set;
+      const size_t ip = set.add(pp.data(), pp.size()), io = set.add(poff.data(), poff.size()),
+                   it = set.add(toff.data(), toff.size());
+      TRY(m->stage.push_all(set));
+      const PackedProb* dpp = set.ptr<PackedProb>(ip);
+      const long long *dpo = set.ptr<long long>(io), *dto = set.ptr<long long>(it);
       m->prof.tc[kind] += 1;
       CUDA_TRY(launch_tc_packed(dpp, dpo, dto, np, poff.back(), toff.back(), m->tc_err, m->stream));
       i0 = i1;
@@ -707,10 +820,11 @@ static int launch_gemm_group(ctebd_mps* m, const std::vector<GemmProb>& probs, i
   }
   std::vector<long long> off(probs.size() + 1, 0);
   for (size_t i = 0; i < probs.size(); i++) off[i + 1] = off[i] + gemm_tiles(probs[i], m->fp64);
-  const GemmProb* dp;
-  const long long* doff;
-  TRY(m->stage.push(probs.data(), probs.size(), &dp));
-  TRY(m->stage.push(off.data(), off.size(), &doff));
+  Staging::Set set;
+  const size_t ip = set.add(probs.data(), probs.size()), io = set.add(off.data(), off.size());
+  TRY(m->stage.push_all(set));
+  const GemmProb* dp = set.ptr<GemmProb>(ip);
+  const long long* doff = set.ptr<long long>(io);
   ProfScope ps(m->prof, m->stream, kind, fl, by);
   cudaError_t e = m->fp64 ? launch_gemm<double>(dp, doff, (int)probs.size(), off.back(), m->stream)
                           : launch_gemm<float>(dp, doff, (int)probs.size(), off.back(), m->stream);
@@ -797,8 +911,11 @@ static int carve_work(ctebd_mps* m, std::vector<Work>& ws) {
     m->arena_cap = want;
   }
   unsigned char* p = (unsigned char*)m->arena;
+  for (auto& w : ws)   // the results of all items side by side
+    w.res = reinterpret_cast<double*>(p), p += 256;
   for (auto& w : ws)
     for (auto& pb : work_buffers(m, w)) {
+      if (pb.first == (void**)&w.res) continue;
       *pb.first = p;
       p += al(pb.second);
     }
@@ -808,7 +925,7 @@ static int carve_work(ctebd_mps* m, std::vector<Work>& ws) {
 static int alloc_owned(ctebd_mps* m, Work& w) {
   work_sizes(m, w);
   for (auto& pb : work_buffers(m, w))
-    if (cudaMallocAsync(pb.first, std::max<size_t>(pb.second, 16), m->stream) != cudaSuccess)
+    if (pool_alloc(m, pb.first, std::max<size_t>(pb.second, 16)) != cudaSuccess)
       return fail(CTEBD_ERR_OOM, "work buffer");
   w.owned = true;
   return CTEBD_OK;
@@ -846,52 +963,75 @@ static int merge_apply(ctebd_mps* m, std::vector<Work>& ws, const std::vector<co
     }
     TRY(run_gemms(m, probs, KK_GEMM_MERGE));
   }
-  // U (host c128) -> device run precision, then theta' = U theta per left index
+  // U (host c128) in run precision, then theta' = U theta per left index: a small cluster's U goes to the device
+  // with the descriptors (at most kApplyGroup clusters to a launch), a large one's into the J scratch
+  constexpr size_t kApplyGroup = 256;
   std::vector<GemmProb> probs;
-  std::vector<ApplyUProb> small;
+  std::vector<float> u32;
+  auto in_run_precision = [&](const double* U, size_t count) -> const void* {
+    if (m->fp64) return U;
+    u32.resize(2 * count);
+    for (size_t e = 0; e < 2 * count; e++) u32[e] = (float)U[e];
+    return u32.data();
+  };
+  struct Small { ApplyUProb u; size_t at; };
+  std::vector<Small> small;
+  Staging::Set set;
   long long max_cols = 0;
   double u_flops = 0, u_bytes = 0;
+  auto flush_small = [&]() -> int {
+    if (small.empty()) return CTEBD_OK;
+    // the U's places are known once the set has its place on the device: their offsets first, then the descriptors
+    size_t at;
+    const size_t head = (set.bytes.size() + 15) & ~size_t(15), bytes = head + small.size() * sizeof(ApplyUProb);
+    TRY(m->stage.room(bytes, &at));
+    std::memcpy(m->stage.h + at, set.bytes.data(), set.bytes.size());
+    for (size_t i = 0; i < small.size(); i++) {
+      small[i].u.U = m->stage.d + at + small[i].at;
+      std::memcpy(m->stage.h + at + head + i * sizeof(ApplyUProb), &small[i].u, sizeof(ApplyUProb));
+    }
+    CUDA_TRY(cudaMemcpyAsync(m->stage.d + at, m->stage.h + at, bytes, cudaMemcpyHostToDevice, m->stream));
+    const ApplyUProb* dsu = reinterpret_cast<const ApplyUProb*>(m->stage.d + at + head);
+    ProfScope ps(m->prof, m->stream, KK_GEMM_U, u_flops, u_bytes);
+    CUDA_TRY(m->fp64 ? launch_apply_u<double>(dsu, (int)small.size(), max_cols, m->stream)
+                     : launch_apply_u<float>(dsu, (int)small.size(), max_cols, m->stream));
+    small.clear();
+    set.bytes.clear();
+    max_cols = 0;
+    u_flops = u_bytes = 0;
+    return CTEBD_OK;
+  };
   for (size_t i = 0; i < ws.size(); i++) {
     Work& w = ws[i];
     const long long D = 1LL << w.k;
-    const double* dU;
-    TRY(m->stage.push(Us[i], (size_t)(2 * D * D), &dU));
+    if ((size_t)(16 * D * D) > Staging::kMax) return fail(CTEBD_ERR_OOM, "staging buffer too small");
+    const void* Uh = in_run_precision(Us[i], (size_t)(D * D));
     void* src = cur[i] ? cur[i] : m->site[w.q0];
-    // convert U into the spare half of the non-source buffer's tail: use J scratch
-    void* Ud = w.J;
-    if ((size_t)(D * D) > w.jElems) return fail(CTEBD_ERR_ARG, "cluster too large for U scratch");
-    cudaError_t e = m->fp64 ? launch_convert_from_c128<double>(dU, Ud, D * D, m->stream)
-                            : launch_convert_from_c128<float>(dU, Ud, D * D, m->stream);
-    CUDA_TRY(e);
     void* dst = (src == w.bufA) ? w.bufB : w.bufA;
+    // keep theta' in bufA: swap the roles of the two buffers for this work item
+    if (dst != w.bufA) std::swap(w.bufA, w.bufB);
     if (D <= 16) {   // small clusters: streaming transform of the (a, b) columns
-      ApplyUProb u{};
-      u.U = Ud; u.src = src; u.dst = dst; u.chiL = w.chiL; u.chiR = w.chiR; u.D = (int)D;
+      Small u{};
+      u.at = set.add(static_cast<const unsigned char*>(Uh), (size_t)(D * D) * m->esz);
+      u.u.src = src; u.u.dst = dst; u.u.chiL = w.chiL; u.u.chiR = w.chiR; u.u.D = (int)D;
       small.push_back(u);
       max_cols = std::max(max_cols, (long long)w.chiL * w.chiR);
       u_flops += 8.0 * D * D * w.chiL * (double)w.chiR;
       u_bytes += 2.0 * D * w.chiL * (double)w.chiR * m->esz;
-      if (dst != w.bufA) std::swap(w.bufA, w.bufB);
+      if (small.size() == kApplyGroup) TRY(flush_small());
       continue;
     }
+    void* Ud = w.J;
+    if ((size_t)(D * D) > w.jElems) return fail(CTEBD_ERR_ARG, "cluster too large for U scratch");
+    TRY(m->stage.copy_to(Ud, Uh, (size_t)(D * D) * m->esz));
     GemmProb p{};
     p.M = (int)D; p.N = w.chiR; p.K = (int)D; p.batch = w.chiL;
     p.A = Ud; p.lda = (int)D; p.opA = 0; p.sA = 0;
     p.B = src; p.ldb = w.chiR; p.opB = 0; p.sB = D * w.chiR;
     p.C = dst; p.ldc = w.chiR; p.sC = D * w.chiR; p.alpha = 1.0;
     probs.push_back(p);
-    if (dst != w.bufA) {
-      // keep theta' in bufA: swap the roles of the two buffers for this work item
-      std::swap(w.bufA, w.bufB);
-    }
   }
-  if (!small.empty()) {
-    const ApplyUProb* dsu;
-    TRY(m->stage.push(small.data(), small.size(), &dsu));
-    ProfScope ps(m->prof, m->stream, KK_GEMM_U, u_flops, u_bytes);
-    CUDA_TRY(m->fp64 ? launch_apply_u<double>(dsu, (int)small.size(), max_cols, m->stream)
-                     : launch_apply_u<float>(dsu, (int)small.size(), max_cols, m->stream));
-  }
+  TRY(flush_small());
   TRY(run_gemms(m, probs, KK_GEMM_U));
   for (auto& w : ws) w.rdim = w.chiR;
   return CTEBD_OK;
@@ -1318,8 +1458,6 @@ static int level_project_select(ctebd_mps* m, std::vector<Work>& ws, const Level
     p.B = w.V; p.ldb = L.vld[a]; p.opB = 0;
     p.C = w.bufB; p.ldc = L.ne[a]; p.alpha = 1.0;
     probs.push_back(p);
-    CUDA_TRY(cudaMemsetAsync(w.rho, 0, sizeof(double) * L.ne[a], m->stream));
-    CUDA_TRY(cudaMemsetAsync(w.rho + w.nmax, 0, sizeof(double) * L.ne[a], m->stream));
     max_n = std::max(max_n, L.ne[a]);
     max_m = std::max(max_m, std::max(L.mm[a], L.nn[a]));
   }
@@ -1341,14 +1479,15 @@ static int level_project_select(ctebd_mps* m, std::vector<Work>& ws, const Level
       mm[na + i] = L.nn[a]; nn[na + i] = L.ne[a]; sh[na + i] = 0; ld[na + i] = L.vld[a];
       by += ((double)L.mm[a] + L.nn[a]) * L.ne[a] * m->esz;
     }
-    const void* const* dR; const int *dm, *dn, *dsh, *dld; const double* const* dL; double* const* drho;
-    TRY(m->stage.push(R.data(), 2 * na, (const void* const**)&dR));
-    TRY(m->stage.push(mm.data(), 2 * na, &dm));
-    TRY(m->stage.push(nn.data(), 2 * na, &dn));
-    TRY(m->stage.push(sh.data(), 2 * na, &dsh));
-    TRY(m->stage.push(ld.data(), 2 * na, &dld));
-    TRY(m->stage.push(Lm.data(), 2 * na, (const double* const**)&dL));
-    TRY(m->stage.push(rho.data(), 2 * na, (double* const**)&drho));
+    Staging::Set set;
+    const size_t iR = set.add(R.data(), 2 * na), iL = set.add(Lm.data(), 2 * na), ir = set.add(rho.data(), 2 * na),
+                 im = set.add(mm.data(), 2 * na), in = set.add(nn.data(), 2 * na), is = set.add(sh.data(), 2 * na),
+                 il = set.add(ld.data(), 2 * na);
+    TRY(m->stage.push_all(set));
+    const void* const* dR = set.ptr<const void*>(iR);
+    const double* const* dL = set.ptr<const double*>(iL);
+    double* const* drho = set.ptr<double*>(ir);
+    const int *dm = set.ptr<int>(im), *dn = set.ptr<int>(in), *dsh = set.ptr<int>(is), *dld = set.ptr<int>(il);
     ProfScope ps(m->prof, m->stream, KK_COLNORM, 0, by);
     CUDA_TRY(f64 ? launch_colnorm_batch<double>(dR, dm, dn, dld, dL, dsh, drho, 2 * na, max_n, max_m, m->stream)
                  : launch_colnorm_batch<float>(dR, dm, dn, dld, dL, dsh, drho, 2 * na, max_n, max_m, m->stream));
@@ -1378,15 +1517,19 @@ static int level_project_select(ctebd_mps* m, std::vector<Work>& ws, const Level
     CUDA_TRY(launch_select(dsp, na, m->cfg.chi_max, m->cfg.cutoff, band, resolved, floor_rel * floor_rel,
                            m->stream));
   }
-  // results land at the level-local index a (h_res[16 a .. 16 a + 15])
   int* h_flag = reinterpret_cast<int*>(m->h_res + 16 * m->h_res_cap);
   *h_flag = 0;
   if (L.act.size() > m->h_res_cap) return fail(CTEBD_ERR_ARG, "too many clusters");
-  for (int a : sel)
-    CUDA_TRY(cudaMemcpyAsync(m->h_res + 16 * a, ws[L.act[a]].res, 16 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+  // the work items' results lie 256 bytes apart: one copy from the first to the last of the selection
+  int lo = L.act[sel[0]], hi = lo;
+  for (int a : sel) { lo = std::min(lo, L.act[a]); hi = std::max(hi, L.act[a]); }
+  CUDA_TRY(cudaMemcpy2DAsync(m->h_raw, 16 * sizeof(double), ws[lo].res, 256, 16 * sizeof(double), hi - lo + 1,
+                             cudaMemcpyDeviceToHost, m->stream));
   if (m->tc_err) CUDA_TRY(cudaMemcpyAsync(h_flag, m->tc_err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
   CUDA_TRY(cudaStreamSynchronize(m->stream));
   m->stage.reset();
+  // by level-local index: h_res[16 a .. 16 a + 15]
+  for (int a : sel) std::memcpy(m->h_res + 16 * a, m->h_raw + 16 * (L.act[a] - lo), 16 * sizeof(double));
   if (*h_flag) return check_tc_flag(m);
   return CTEBD_OK;
 }
@@ -1800,23 +1943,9 @@ static bool use_small(const ctebd_mps* m, const Work& w, size_t& smem) {
 // are read by small_finish, after other work has been queued.
 static int small_start(ctebd_mps* m, std::vector<Work>& ws, const std::vector<int>& sel, size_t smem) {
   std::vector<SmallProb> sp(sel.size());
-  size_t rows = 0;
+  size_t rows = 0;                 // fewer than the qubits
   double fl = 0;
   for (int i : sel) rows += ws[i].k - 1;
-  if (8 * rows > m->small_cap) {   // device results and their pinned copy
-    CUDA_TRY(cudaStreamSynchronize(m->stream));
-    if (m->small_res) CUDA_TRY(cudaFree(m->small_res));
-    if (m->h_small) CUDA_TRY(cudaFreeHost(m->h_small));
-    m->small_res = m->h_small = nullptr;
-    m->small_cap = 0;
-    const size_t want = 8 * (rows + rows / 2 + 64);
-    if (cudaMalloc(&m->small_res, want * sizeof(double)) != cudaSuccess ||
-        cudaMallocHost(&m->h_small, want * sizeof(double)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(CTEBD_ERR_OOM, "split results");
-    }
-    m->small_cap = want;
-  }
   double* res = m->small_res;
   for (size_t a = 0; a < sel.size(); a++) {
     Work& w = ws[sel[a]];
@@ -1977,7 +2106,9 @@ static int split_levels(ctebd_mps* m, std::vector<Work>& ws, std::vector<std::ve
       g0.cs = w.rho + w.nmax;
       gp.push_back(g0);
       GatherProb g1{};
-      g1.src = w.bufB; g1.dst = w.bufA; g1.perm = w.perm; g1.rows = L.mm[a]; g1.r = r; g1.ld = L.ne[a]; g1.mode = 1;
+      // the remainder: the next level's matrix, or the leftmost site
+      if (j == 1) TRY(ensure_site(m, w.q0, (size_t)L.mm[a] * r));
+      g1.src = w.bufB; g1.dst = j == 1 ? m->site[w.q0] : w.bufA; g1.perm = w.perm; g1.rows = L.mm[a]; g1.r = r; g1.ld = L.ne[a]; g1.mode = 1;
       g1.scale = 1.0 / std::sqrt(kept);
       g1.cs = w.rho + w.nmax;
       gp.push_back(g1);
@@ -2005,14 +2136,6 @@ static int split_levels(ctebd_mps* m, std::vector<Work>& ws, std::vector<std::ve
     fs[r.i].push_back(r.row[6]);
     m->splitlog.insert(m->splitlog.end(), r.row, r.row + 8);
     m->splitlog2.insert(m->splitlog2.end(), r.row + 8, r.row + 14);
-  }
-  // leftmost site of every other cluster: the remainder (chiL*2 x r1)
-  for (size_t i = 0; i < ws.size(); i++) {
-    Work& w = ws[i];
-    if (is_small[i]) continue;
-    const size_t elems = (size_t)w.chiL * 2 * w.rdim;
-    TRY(ensure_site(m, w.q0, elems));
-    CUDA_TRY(cudaMemcpyAsync(m->site[w.q0], w.bufA, elems * m->esz, cudaMemcpyDeviceToDevice, m->stream));
   }
   return CTEBD_OK;
 }
@@ -2109,11 +2232,12 @@ extern "C" int apply_1q(ctebd_mps* m, int q, const double* u) {
   CUDA_TRY(cudaStreamSynchronize(m->stream));
   void* s = m->site[q];
   const int cl = m->chi[q], cr = m->chi[q + 1];
-  void* const* ds; const int *dcl, *dcr; const double* du;
-  TRY(m->stage.push(&s, 1, (void* const**)&ds));
-  TRY(m->stage.push(&cl, 1, &dcl));
-  TRY(m->stage.push(&cr, 1, &dcr));
-  TRY(m->stage.push(u, 8, &du));
+  Staging::Set set;
+  const size_t is = set.add(&s, 1), iu = set.add(u, 8), il = set.add(&cl, 1), ir = set.add(&cr, 1);
+  TRY(m->stage.push_all(set));
+  void* const* ds = set.ptr<void*>(is);
+  const int *dcl = set.ptr<int>(il), *dcr = set.ptr<int>(ir);
+  const double* du = set.ptr<double>(iu);
   {
     ProfScope ps(m->prof, m->stream, KK_ONEQ, 28.0 * cl * cr, 4.0 * cl * cr * m->esz);
     CUDA_TRY(m->fp64 ? launch_apply_1q<double>(ds, dcl, dcr, du, 1, (long long)cl * cr, m->stream)
@@ -2166,11 +2290,13 @@ extern "C" int apply_singletons(ctebd_mps* m, const ctebd_gate* gates, int n_gat
   }
   CUDA_TRY(cudaStreamSynchronize(m->stream));
   m->stage.reset();
-  void* const* ds; const int *dcl, *dcr; const double* du;
-  TRY(m->stage.push(sites.data(), sites.size(), (void* const**)&ds));
-  TRY(m->stage.push(cls.data(), cls.size(), &dcl));
-  TRY(m->stage.push(crs.data(), crs.size(), &dcr));
-  TRY(m->stage.push(us.data(), us.size(), &du));
+  Staging::Set set;
+  const size_t is = set.add(sites.data(), sites.size()), iu = set.add(us.data(), us.size()),
+               il = set.add(cls.data(), cls.size()), ir = set.add(crs.data(), crs.size());
+  TRY(m->stage.push_all(set));
+  void* const* ds = set.ptr<void*>(is);
+  const int *dcl = set.ptr<int>(il), *dcr = set.ptr<int>(ir);
+  const double* du = set.ptr<double>(iu);
   double e1 = 0;
   for (size_t i = 0; i < sites.size(); i++) e1 += (double)cls[i] * crs[i];
   {
@@ -2236,11 +2362,29 @@ extern "C" int mps_to_host(const ctebd_mps* mc, int q, double* buf, size_t cap) 
   if (!m || !buf || q < 0 || q >= m->n) return fail(CTEBD_ERR_ARG, "mps_to_host: bad args");
   const long long n = (long long)m->chi[q] * 2 * m->chi[q + 1];
   if ((size_t)(2 * n) > cap) return fail(CTEBD_ERR_ARG, "mps_to_host: buffer too small");
+  // FP64 sites are c128 already.  FP32: widened on the host up to 128 KB (copy 9 us, loop 4), above that by a kernel
+  // (256 KB: 12 us on the host, 10 + 12 by kernel and copy; 1 MB: 78 against 44), in pieces of 64 MB
+  if (m->fp64) {
+    CUDA_TRY(cudaMemcpyAsync(buf, m->site[q], sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, m->stream));
+    CUDA_TRY(cudaStreamSynchronize(m->stream));
+    return CTEBD_OK;
+  }
+  const float* src = static_cast<const float*>(m->site[q]);
+  if (n <= 16384) {
+    std::vector<float> f(2 * n);
+    CUDA_TRY(cudaMemcpyAsync(f.data(), src, sizeof(float) * 2 * n, cudaMemcpyDeviceToHost, m->stream));
+    CUDA_TRY(cudaStreamSynchronize(m->stream));
+    for (long long i = 0; i < 2 * n; i++) buf[i] = f[i];
+    return CTEBD_OK;
+  }
+  const long long piece = std::min<long long>(n, 1 << 22);
   double* d = nullptr;
-  CUDA_TRY(cudaMallocAsync(&d, sizeof(double) * 2 * n, m->stream));
-  CUDA_TRY(m->fp64 ? launch_convert_to_c128<double>(m->site[q], d, n, m->stream)
-                   : launch_convert_to_c128<float>(m->site[q], d, n, m->stream));
-  CUDA_TRY(cudaMemcpyAsync(buf, d, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, m->stream));
+  CUDA_TRY(pool_alloc(m, &d, sizeof(double) * 2 * piece));
+  for (long long i = 0; i < n; i += piece) {
+    const long long c = std::min(piece, n - i);
+    CUDA_TRY(launch_widen_c128(src + 2 * i, d, c, m->stream));
+    CUDA_TRY(cudaMemcpyAsync(buf + 2 * i, d, sizeof(double) * 2 * c, cudaMemcpyDeviceToHost, m->stream));
+  }
   CUDA_TRY(cudaFreeAsync(d, m->stream));
   CUDA_TRY(cudaStreamSynchronize(m->stream));
   return CTEBD_OK;
@@ -2269,13 +2413,15 @@ extern "C" int mps_load(ctebd_mps* m, const int* chi, const double* const* sites
   for (int q = 0; q < m->n; q++) {
     const long long n = (long long)chi[q] * 2 * chi[q + 1];
     TRY(ensure_site(m, q, (size_t)n));
+    if (m->fp64) {
+      CUDA_TRY(cudaMemcpyAsync(m->site[q], sites[q], sizeof(double) * 2 * n, cudaMemcpyHostToDevice, m->stream));
+      continue;
+    }
     double* d = nullptr;
-    CUDA_TRY(cudaMallocAsync(&d, sizeof(double) * 2 * n, m->stream));
+    CUDA_TRY(pool_alloc(m, &d, sizeof(double) * 2 * n));
     CUDA_TRY(cudaMemcpyAsync(d, sites[q], sizeof(double) * 2 * n, cudaMemcpyHostToDevice, m->stream));
-    CUDA_TRY(m->fp64 ? launch_convert_from_c128<double>(d, m->site[q], n, m->stream)
-                     : launch_convert_from_c128<float>(d, m->site[q], n, m->stream));
+    CUDA_TRY(launch_narrow_c128(d, static_cast<float*>(m->site[q]), n, m->stream));
     CUDA_TRY(cudaFreeAsync(d, m->stream));
-    CUDA_TRY(cudaStreamSynchronize(m->stream));
   }
   for (int b = 0; b <= m->n; b++)
     CUDA_TRY(cudaMemcpyAsync(m->lam[b], lams[b], sizeof(double) * chi[b], cudaMemcpyHostToDevice, m->stream));
@@ -2288,13 +2434,36 @@ extern "C" int mps_load(ctebd_mps* m, const int* chi, const double* const* sites
 extern "C" int mps_load_device(ctebd_mps* m, const int* chi, const void* const* sites, const double* const* lams) {
   if (!m || !chi || !sites || !lams) return fail(CTEBD_ERR_ARG, "mps_load_device: null argument");
   TRY(check_chi(m, chi));
+  // This device's own memory in one launch (4 us a copy otherwise); host or other memory, and what is not aligned to
+  // an element, by its own copy.
+  int dev = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  std::vector<CopyProb> cp;
+  size_t largest = 0;
+  auto add = [&](void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) -> int {
+    cudaPointerAttributes at{};
+    const bool known = cudaPointerGetAttributes(&at, src) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    if (known && at.type == cudaMemoryTypeDevice && at.device == dev && reinterpret_cast<uintptr_t>(src) % 8 == 0) {
+      cp.push_back({src, dst, (long long)(bytes / 8)});
+      largest = std::max(largest, bytes / 8);
+      return CTEBD_OK;
+    }
+    CUDA_TRY(cudaMemcpyAsync(dst, src, bytes, kind, m->stream));
+    return CTEBD_OK;
+  };
   for (int q = 0; q < m->n; q++) {
     const size_t n = (size_t)chi[q] * 2 * chi[q + 1];
     TRY(ensure_site(m, q, n));
-    CUDA_TRY(cudaMemcpyAsync(m->site[q], sites[q], n * m->esz, cudaMemcpyDeviceToDevice, m->stream));
+    TRY(add(m->site[q], sites[q], n * m->esz, cudaMemcpyDeviceToDevice));
   }
-  for (int b = 0; b <= m->n; b++)
-    CUDA_TRY(cudaMemcpyAsync(m->lam[b], lams[b], sizeof(double) * chi[b], cudaMemcpyDefault, m->stream));
+  for (int b = 0; b <= m->n; b++) TRY(add(m->lam[b], lams[b], sizeof(double) * chi[b], cudaMemcpyDefault));
+  if (!cp.empty()) {
+    m->stage.reset();   // every call has waited for the stream before it returned
+    const CopyProb* dc;
+    TRY(m->stage.push(cp.data(), cp.size(), &dc));
+    CUDA_TRY(launch_copy_batch(dc, (int)cp.size(), (long long)largest, m->stream));
+  }
   m->chi.assign(chi, chi + m->n + 1);
   m->logF = 0;
   CUDA_TRY(cudaStreamSynchronize(m->stream));
@@ -2563,7 +2732,7 @@ extern "C" int mps_bond_entropies(ctebd_mps* m, double* out) {
   if (!m || !out) return fail(CTEBD_ERR_ARG, "mps_bond_entropies: null argument");
   const int nb = m->n + 1;
   double* d = nullptr;
-  CUDA_TRY(cudaMallocAsync(&d, sizeof(double) * nb, m->stream));
+  CUDA_TRY(pool_alloc(m, &d, sizeof(double) * nb));
   const double* const* dl; const int* dc;
   CUDA_TRY(cudaStreamSynchronize(m->stream));
   m->stage.reset();
@@ -2594,8 +2763,8 @@ extern "C" int rank_model_predict(ctebd_mps* m, const float* features, int B, co
   if (!m->mlp) return fail(CTEBD_ERR_STATE, "rank_model_predict: no model loaded");
   if (B == 0) return CTEBD_OK;
   float *dX = nullptr, *dL = nullptr;
-  CUDA_TRY(cudaMallocAsync(&dX, sizeof(float) * B * MLP_F, m->stream));
-  CUDA_TRY(cudaMallocAsync(&dL, sizeof(float) * B * MLP_NB, m->stream));
+  CUDA_TRY(pool_alloc(m, &dX, sizeof(float) * B * MLP_F));
+  CUDA_TRY(pool_alloc(m, &dL, sizeof(float) * B * MLP_NB));
   CUDA_TRY(cudaMemcpyAsync(dX, features, sizeof(float) * B * MLP_F, cudaMemcpyHostToDevice, m->stream));
   {
     ProfScope ps(m->prof, m->stream, KK_MLP, 2.0 * B * (MLP_F * MLP_H1 + MLP_H1 * MLP_H2 + MLP_H2 * MLP_NB), 0);

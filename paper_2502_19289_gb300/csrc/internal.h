@@ -270,10 +270,16 @@ size_t amp_scratch_bytes(int max_chi);
 template <typename R>
 cudaError_t launch_amplitude(const AmpSite* d_sites, int n, int mid_chi, int max_chi, int ctas, unsigned char* scratch,
                              double2* out, int* err, cudaStream_t s);
-template <typename R>
-cudaError_t launch_convert_from_c128(const double* src, void* dst, long long n, cudaStream_t s);
-template <typename R>
-cudaError_t launch_convert_to_c128(const void* src, double* dst, long long n, cudaStream_t s);
+cudaError_t launch_narrow_c128(const double* src, float* dst, long long n, cudaStream_t s);   // n complex numbers
+cudaError_t launch_widen_c128(const float* src, double* dst, long long n, cudaStream_t s);
+
+// words of 8 bytes (src and dst 8-byte aligned)
+struct CopyProb {
+  const void* src;
+  void* dst;
+  long long words;
+};
+cudaError_t launch_copy_batch(const CopyProb* d_probs, int count, long long max_words, cudaStream_t s);
 
 // rank predictor network (features -> hidden -> hidden -> rank buckets)
 constexpr int MLP_F = 16, MLP_H1 = 64, MLP_H2 = 64, MLP_NB = 16;

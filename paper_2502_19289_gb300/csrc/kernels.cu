@@ -1247,42 +1247,56 @@ template cudaError_t launch_apply_1q<float>(void* const*, const int*, const int*
 template cudaError_t launch_apply_1q<double>(void* const*, const int*, const int*, const double*,
                                              int, long long, cudaStream_t);
 
-template <typename R>
-__global__ void k_from_c128(const double* __restrict__ src, void* __restrict__ dst, long long n) {
-  using CT = typename C2<R>::T;
-  CT* d = (CT*)dst;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    d[i] = cmk<CT>(src[2 * i], src[2 * i + 1]);
-}
-template <typename R>
-__global__ void k_to_c128(const void* __restrict__ src, double* __restrict__ dst, long long n) {
-  using CT = typename C2<R>::T;
-  const CT* s = (const CT*)src;
+// FP32 complex <-> complex128
+__global__ void k_narrow_c128(const double2* __restrict__ src, float2* __restrict__ dst, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    dst[2 * i] = s[i].x;
-    dst[2 * i + 1] = s[i].y;
+    const double2 v = src[i];
+    dst[i] = make_float2((float)v.x, (float)v.y);
   }
 }
-template <typename R>
-cudaError_t launch_convert_from_c128(const double* src, void* dst, long long n, cudaStream_t s) {
+__global__ void k_widen_c128(const float2* __restrict__ src, double2* __restrict__ dst, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const float2 v = src[i];
+    dst[i] = make_double2(v.x, v.y);
+  }
+}
+cudaError_t launch_narrow_c128(const double* src, float* dst, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  long long g = (n + 255) / 256;
-  k_from_c128<R><<<(unsigned)(g > 8192 ? 8192 : g), 256, 0, s>>>(src, dst, n);
+  const long long g = (n + 255) / 256;
+  k_narrow_c128<<<(unsigned)(g > 8192 ? 8192 : g), 256, 0, s>>>((const double2*)src, (float2*)dst, n);
   return cudaGetLastError();
 }
-template <typename R>
-cudaError_t launch_convert_to_c128(const void* src, double* dst, long long n, cudaStream_t s) {
+cudaError_t launch_widen_c128(const float* src, double* dst, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  long long g = (n + 255) / 256;
-  k_to_c128<R><<<(unsigned)(g > 8192 ? 8192 : g), 256, 0, s>>>(src, dst, n);
+  const long long g = (n + 255) / 256;
+  k_widen_c128<<<(unsigned)(g > 8192 ? 8192 : g), 256, 0, s>>>((const float2*)src, (double2*)dst, n);
   return cudaGetLastError();
 }
-template cudaError_t launch_convert_from_c128<float>(const double*, void*, long long, cudaStream_t);
-template cudaError_t launch_convert_from_c128<double>(const double*, void*, long long, cudaStream_t);
-template cudaError_t launch_convert_to_c128<float>(const void*, double*, long long, cudaStream_t);
-template cudaError_t launch_convert_to_c128<double>(const void*, double*, long long, cudaStream_t);
+
+// Several device buffers in one launch, 16 bytes a thread where both ends
+// allow it.  A state of 48 tensors and 49 spectra: 97 copies of 4 us each.
+__global__ void __launch_bounds__(256) k_copy_batch(const CopyProb* __restrict__ probs) {
+  const CopyProb P = probs[blockIdx.y];
+  const long long t0 = blockIdx.x * 256LL + threadIdx.x, step = gridDim.x * 256LL;
+  if ((((uintptr_t)P.src | (uintptr_t)P.dst) & 15) == 0) {
+    const uint4* a = (const uint4*)P.src;
+    uint4* b = (uint4*)P.dst;
+    for (long long i = t0; i < P.words / 2; i += step) b[i] = a[i];
+    if ((P.words & 1) && t0 == 0) ((uint2*)P.dst)[P.words - 1] = ((const uint2*)P.src)[P.words - 1];
+  } else {
+    for (long long i = t0; i < P.words; i += step) ((uint2*)P.dst)[i] = ((const uint2*)P.src)[i];
+  }
+}
+cudaError_t launch_copy_batch(const CopyProb* d_probs, int count, long long max_words, cudaStream_t s) {
+  long long gx = (max_words / 2 + 1023) / 1024;
+  if (gx > 1024) gx = 1024;
+  if (gx < 1) gx = 1;
+  for (int i = 0; i < count; i += 32768)
+    k_copy_batch<<<dim3((unsigned)gx, (unsigned)(count - i < 32768 ? count - i : 32768)), 256, 0, s>>>(d_probs + i);
+  return cudaGetLastError();
+}
 
 // ---------------------------------------------------------------------------
 // FP32 FMA throughput probe (the CUDA-core roofline of the FP32 kernels):
