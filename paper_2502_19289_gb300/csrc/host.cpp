@@ -819,15 +819,16 @@ static int launch_gemm_group(ctebd_mps* m, const std::vector<GemmProb>& probs, i
     return CTEBD_OK;
   }
   std::vector<long long> off(probs.size() + 1, 0);
-  for (size_t i = 0; i < probs.size(); i++) off[i + 1] = off[i] + gemm_tiles(probs[i], m->fp64);
+  const int tm = gemm_tile(probs.data(), (int)probs.size(), m->fp64);
+  for (size_t i = 0; i < probs.size(); i++) off[i + 1] = off[i] + gemm_tiles(probs[i], tm);
   Staging::Set set;
   const size_t ip = set.add(probs.data(), probs.size()), io = set.add(off.data(), off.size());
   TRY(m->stage.push_all(set));
   const GemmProb* dp = set.ptr<GemmProb>(ip);
   const long long* doff = set.ptr<long long>(io);
   ProfScope ps(m->prof, m->stream, kind, fl, by);
-  cudaError_t e = m->fp64 ? launch_gemm<double>(dp, doff, (int)probs.size(), off.back(), m->stream)
-                          : launch_gemm<float>(dp, doff, (int)probs.size(), off.back(), m->stream);
+  cudaError_t e = m->fp64 ? launch_gemm<double>(dp, doff, (int)probs.size(), off.back(), tm, m->stream)
+                          : launch_gemm<float>(dp, doff, (int)probs.size(), off.back(), tm, m->stream);
   CUDA_TRY(e);
   return CTEBD_OK;
 }

@@ -195,9 +195,10 @@ struct GatherProb {
 // Launchers (R = float or double).  Descriptor arrays are device pointers.
 template <typename R>
 cudaError_t launch_gemm(const GemmProb* d_probs, const long long* d_tile_off, int n_probs,
-                        long long total_tiles, cudaStream_t s);
-// tile bookkeeping helper (host): tiles of a problem in the GEMM grid
-long long gemm_tiles(const GemmProb& p, bool fp64);
+                        long long total_tiles, int tm, cudaStream_t s);
+// host: the tile (16 tm x 16 tm) for a group of problems, and a problem's tiles in the grid
+int gemm_tile(const GemmProb* probs, int n, bool fp64);
+long long gemm_tiles(const GemmProb& p, int tm);
 
 template <typename R>
 cudaError_t launch_eig_init(const EigProb* d_probs, int n_probs, int max_npad, cudaStream_t s);

@@ -38,17 +38,19 @@ template <typename T> __device__ __forceinline__ T cscale(T a, double s) {
 }
 
 // ---------------------------------------------------------------------------
-// Grouped complex GEMM, 64x64 output tile, 256 threads (4x4 per thread).
+// Grouped complex GEMM: output tiles of 16 TM x 16 TM, 256 threads with TM x TM
+// elements each, the next slice of K loaded while the present one is used.
 // Merge chain (theta), U application, Gram matrix and Mbar*V all use it.
+// Sums run over k in the same order whatever the tile.
 // ---------------------------------------------------------------------------
-constexpr int GBM = 64, GBN = 64, GBK = 16;
-
-template <typename R>
+template <typename R, int TM>
 __global__ void __launch_bounds__(256) k_gemm(const GemmProb* __restrict__ probs,
                                               const long long* __restrict__ tile_off, int n_probs) {
   using CT = typename C2<R>::T;
-  __shared__ CT As[GBK][GBM + 1];
-  __shared__ CT Bs[GBK][GBN + 1];
+  constexpr int BM = 16 * TM, BK = TM == 4 ? (sizeof(R) == 8 ? 8 : 16) : TM == 2 ? (sizeof(R) == 8 ? 16 : 32) : 32;
+  constexpr int PER = BM * BK / 256;
+  __shared__ CT As[2][BK][BM + 1];
+  __shared__ CT Bs[2][BK][BM + 1];
   const long long tid_tile = blockIdx.x;
   int lo = 0, hi = n_probs;
   while (hi - lo > 1) {
@@ -57,7 +59,7 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmProb* __restrict__ probs
   }
   const GemmProb P = probs[lo];
   long long t = tid_tile - tile_off[lo];
-  const int tilesN = (P.N + GBN - 1) / GBN, tilesM = (P.M + GBM - 1) / GBM;
+  const int tilesN = (P.N + BM - 1) / BM, tilesM = (P.M + BM - 1) / BM;
   const int tn = (int)(t % tilesN);
   t /= tilesN;
   const int tm = (int)(t % tilesM);
@@ -65,83 +67,117 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmProb* __restrict__ probs
   const CT* A = (const CT*)P.A + bidx * P.sA;
   const CT* B = (const CT*)P.B + bidx * P.sB;
   CT* Cm = (CT*)P.C + bidx * P.sC;
-  const int m0 = tm * GBM, n0 = tn * GBN;
+  const int m0 = tm * BM, n0 = tn * BM;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  CT acc[4][4];
+  CT acc[TM][TM], ra[PER], rb[PER];
 #pragma unroll
-  for (int i = 0; i < 4; i++)
+  for (int i = 0; i < TM; i++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = cmk<CT>(0, 0);
-  for (int k0 = 0; k0 < P.K; k0 += GBK) {
+    for (int j = 0; j < TM; j++) acc[i][j] = cmk<CT>(0, 0);
+  // element e of a slice: k fastest where k is contiguous in memory, else the tile's row (column)
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int it = 0; it < 4; it++) {
+    for (int it = 0; it < PER; it++) {
       const int e = threadIdx.x + it * 256;
-      int m, kk;
+      const int m = P.opA == 0 ? e / BK : e % BM, ka = k0 + (P.opA == 0 ? e % BK : e / BM);
       CT v = cmk<CT>(0, 0);
-      if (P.opA == 0) {
-        m = e / GBK; kk = e % GBK;
-        if (m0 + m < P.M && k0 + kk < P.K) v = A[(long long)(m0 + m) * P.lda + k0 + kk];
-      } else {
-        kk = e / GBM; m = e % GBM;
-        if (m0 + m < P.M && k0 + kk < P.K) v = cconj(A[(long long)(k0 + kk) * P.lda + m0 + m]);
+      if (m0 + m < P.M && ka < P.K) {
+        v = P.opA == 0 ? A[(long long)(m0 + m) * P.lda + ka] : cconj(A[(long long)ka * P.lda + m0 + m]);
+        if (P.kw) {
+          const double wk = P.kw[ka >> P.kw_shift];
+          v = cscale(v, P.kw_pow == 1 ? wk : wk * wk);
+        }
       }
-      if (P.kw && k0 + kk < P.K) {
-        const double wk = P.kw[(k0 + kk) >> P.kw_shift];
-        v = cscale(v, P.kw_pow == 1 ? wk : wk * wk);
-      }
-      As[kk][m] = v;
-      int n;
+      ra[it] = v;
+      const int n = P.opB == 0 ? e % BM : e / BK, kb = k0 + (P.opB == 0 ? e / BM : e % BK);
       CT w = cmk<CT>(0, 0);
-      if (P.opB == 0) {
-        kk = e / GBN; n = e % GBN;
-        if (n0 + n < P.N && k0 + kk < P.K) w = B[(long long)(k0 + kk) * P.ldb + n0 + n];
-      } else {
-        n = e / GBK; kk = e % GBK;
-        if (n0 + n < P.N && k0 + kk < P.K) w = cconj(B[(long long)(n0 + n) * P.ldb + k0 + kk]);
-      }
-      Bs[kk][n] = w;
+      if (n0 + n < P.N && kb < P.K)
+        w = P.opB == 0 ? B[(long long)kb * P.ldb + n0 + n] : cconj(B[(long long)(n0 + n) * P.ldb + kb]);
+      rb[it] = w;
     }
-    __syncthreads();
+  };
+  auto store = [&](int buf) {
 #pragma unroll
-    for (int kk = 0; kk < GBK; kk++) {
-      CT a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) cfma(acc[i][j], a[i], b[j]);
+    for (int it = 0; it < PER; it++) {
+      const int e = threadIdx.x + it * 256;
+      if (P.opA == 0) As[buf][e % BK][e / BK] = ra[it]; else As[buf][e / BM][e % BM] = ra[it];
+      if (P.opB == 0) Bs[buf][e / BM][e % BM] = rb[it]; else Bs[buf][e % BK][e / BK] = rb[it];
     }
+  };
+  fetch(0);
+  store(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < P.K; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < P.K;
+    if (more) fetch(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; kk++) {
+      CT a[TM], b[TM];
+#pragma unroll
+      for (int i = 0; i < TM; i++) a[i] = As[buf][kk][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < TM; j++) b[j] = Bs[buf][kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < TM; i++)
+#pragma unroll
+        for (int j = 0; j < TM; j++) cfma(acc[i][j], a[i], b[j]);
+    }
+    if (more) store(buf ^ 1);
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; i++) {
+  for (int i = 0; i < TM; i++) {
     const int m = m0 + ty + 16 * i;
     if (m >= P.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
+    for (int j = 0; j < TM; j++) {
       const int n = n0 + tx + 16 * j;
       if (n < P.N) Cm[(long long)m * P.ldc + n] = cscale(acc[i][j], P.alpha);
     }
   }
 }
 
-long long gemm_tiles(const GemmProb& p, bool) {
-  return (long long)((p.M + GBM - 1) / GBM) * ((p.N + GBN - 1) / GBN) * p.batch;
+long long gemm_tiles(const GemmProb& p, int tm) {
+  const int bm = 16 * tm;
+  return (long long)((p.M + bm - 1) / bm) * ((p.N + bm - 1) / bm) * p.batch;
+}
+
+// Rule: the tile whose waves over 152 SMs cost least, a wave of 16 TM costing
+// TM^2 (FP32: times 1.3 and 2 for the two smaller ones, which read shared
+// memory more often per product).  Products of the splits are small next to
+// the chip -- FP64 runs at 2 lanes a clock and SM, so every idle SM counts.
+// Merge and projection kernels of a step, tile 64 / 32 / 16: four FP64
+// clusters of 128-wide splits 0.55 + 1.08 / 0.16 + 0.29 / 0.13 + 0.23 ms; eight
+// FP64 30-wide 0.074 + 0.143 / 0.027 + 0.047 / 0.019 + 0.023; sixteen FP32
+// 48-wide 0.065 + 0.092 / 0.051 + 0.058 / 0.038 + 0.058; eight FP32 200-wide
+// 0.087 + 0.147 / 0.074 + 0.138 / 0.092 + 0.162.
+int gemm_tile(const GemmProb* probs, int n, bool fp64) {
+  constexpr long long kSms = 152;
+  int best = 4;
+  double cost = 0;
+  for (int tm = 4; tm >= 1; tm >>= 1) {
+    long long tiles = 0;
+    for (int i = 0; i < n; i++) tiles += gemm_tiles(probs[i], tm);
+    const double c = (double)((tiles + kSms - 1) / kSms) * tm * tm * (fp64 || tm == 4 ? 1.0 : tm == 2 ? 1.3 : 2.0);
+    if (tm == 4 || c < cost) { best = tm; cost = c; }
+  }
+  return best;
 }
 
 template <typename R>
 cudaError_t launch_gemm(const GemmProb* d_probs, const long long* d_tile_off, int n_probs,
-                        long long total_tiles, cudaStream_t s) {
+                        long long total_tiles, int tm, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
   if (total_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_gemm<R><<<(unsigned)total_tiles, 256, 0, s>>>(d_probs, d_tile_off, n_probs);
+  const unsigned grid = (unsigned)total_tiles;
+  if (tm == 4) k_gemm<R, 4><<<grid, 256, 0, s>>>(d_probs, d_tile_off, n_probs);
+  else if (tm == 2) k_gemm<R, 2><<<grid, 256, 0, s>>>(d_probs, d_tile_off, n_probs);
+  else k_gemm<R, 1><<<grid, 256, 0, s>>>(d_probs, d_tile_off, n_probs);
   return cudaGetLastError();
 }
-template cudaError_t launch_gemm<float>(const GemmProb*, const long long*, int, long long, cudaStream_t);
-template cudaError_t launch_gemm<double>(const GemmProb*, const long long*, int, long long, cudaStream_t);
+template cudaError_t launch_gemm<float>(const GemmProb*, const long long*, int, long long, int, cudaStream_t);
+template cudaError_t launch_gemm<double>(const GemmProb*, const long long*, int, long long, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // Batched block-Jacobi eigensolver for Hermitian G (two-sided, parallel

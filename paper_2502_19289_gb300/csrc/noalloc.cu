@@ -104,10 +104,12 @@ static int na_gemm(NaDesc& d, const GemmProb& p) {
   struct One {
     GemmProb p;
     long long off[2];
-  } h = {p, {0, gemm_tiles(p, false)}};
+  } h = {p, {0, 0}};
+  const int tm = gemm_tile(&p, 1, false);
+  h.off[1] = gemm_tiles(p, tm);
   const One* dp;
   if (int rc = d.put(&h, 1, &dp)) return rc;
-  NA_CUDA(launch_gemm<float>(&dp->p, dp->off, 1, h.off[1], d.s));
+  NA_CUDA(launch_gemm<float>(&dp->p, dp->off, 1, h.off[1], tm, d.s));
   return CTEBD_OK;
 }
 
