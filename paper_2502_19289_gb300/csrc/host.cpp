@@ -1623,7 +1623,6 @@ static int level_direct(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
     m->prof.launches[KK_TRIDIAG] += launches - 1;
   }
   ProfScope ps(m->prof, m->stream, KK_BACK, fl_v, 0);
-  m->prof.launches[KK_BACK] += 1;
   CUDA_TRY(launch_dir_back<R>(dd, na, max_n, m->stream));
   return CTEBD_OK;
 }
