@@ -4,9 +4,9 @@
 // Narrow splits are bound by launches, host reads of the ranks and the latency
 // of a dozen short kernels per split, not by arithmetic.  Here a CTA keeps the
 // split matrix in shared memory and, level by level,
-//   - reduces M = diag(lambda_L) Mbar to its triangular factor R by Householder
-//     reflectors (one barrier per column),
-//   - makes the columns of R^H orthogonal by one-sided Jacobi rotations; they
+//   - reduces M = diag(lambda_L) Mbar, where it has more rows than columns, to
+//     its triangular factor R by Householder reflectors (a barrier per column),
+//   - makes the columns of R^H (of M^H) orthogonal by one-sided Jacobi rotations; they
 //     are then sigma_i v_i, so no rotations are accumulated (the scheme of
 //     Drmac and Veselic, SIAM J. Matrix Anal. Appl. 29, 1322 (2008), which
 //     keeps small singular values to relative accuracy),
@@ -15,8 +15,10 @@
 //   - writes the new site and the remainder, which is the next level's matrix.
 // Bound by the FP64 units' issue rate within one CTA (a warp's FP64 instruction
 // holds its unit for 64 cycles): so four warps, one per unit, a half warp per
-// pair of vectors, and the rotation angles in FP32, normalised in FP64.  That
-// took a 16 x 16 split from 0.56 to 0.27 ms.
+// pair of vectors, and the rotation angles in FP32, normalised in FP64 (a
+// 16 x 16 split 0.56 -> 0.27 ms); no QR where it would not shorten the vectors
+// (0.27 -> 0.20).  Splits of a few columns are bound by instruction fetch: 12 us
+// each.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -66,6 +68,13 @@ __device__ __forceinline__ void hsum4(double& a, double& b, double& c, double& d
   d = __shfl_sync(0xffffffffu, u, base + 3);
 }
 
+// largest of K numbers that are not negative, compared as integers
+__device__ __forceinline__ double largest(const double* v, int K) {
+  long long t = 0;
+  for (int i = 0; i < K; i++) t = max(t, __double_as_longlong(v[i]));
+  return __longlong_as_double(t);
+}
+
 __device__ __forceinline__ double2 wide(float2 v) { return make_double2(v.x, v.y); }
 __device__ __forceinline__ double2 wide(double2 v) { return v; }
 
@@ -101,17 +110,20 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     const int ld = m | 1, ldx = n | 1;
     CT* A = reinterpret_cast<CT*>(smraw);            // n columns of m (stride ld), then Z
     CT* X = A + (size_t)n * ld;                      // K vectors of n (stride ldx): columns of R^H
-    // ---- M = diag(lambda) Mbar, column by column
+    // ---- M = diag(lambda) Mbar, column by column; with no more rows than columns the rows are the vectors
+    const bool tall = m > n;
+    if (tall)
+      for (int e = tid; e < K * ldx; e += NT) X[e] = make_double2(0, 0);
     for (int e = tid; e < m * n; e += NT) {
       const int r = e / n, c = e - r * n;
       const CT v = wide(src[e]);
       const double l = P.lam[r >> j];
-      A[c * ld + r] = make_double2(v.x * l, v.y * l);
+      if (tall) A[c * ld + r] = make_double2(v.x * l, v.y * l);
+      else X[r * ldx + c] = make_double2(v.x * l, -v.y * l);
     }
-    for (int e = tid; e < K * ldx; e += NT) X[e] = make_double2(0, 0);
     __syncthreads();
     // ---- R: every half warp reflects column c alike and takes its share of the columns behind it
-    for (int c = 0; c < K; c++) {
+    for (int c = 0; tall && c < K; c++) {
       const CT* a = A + c * ld;
       double s = 0;
       for (int r = c + 1 + c0; r < m; r += 16) s = fma(a[r].x, a[r].x, fma(a[r].y, a[r].y, s));
@@ -153,8 +165,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
       if (c0 == 0) nrm[i] = s;
     }
     __syncthreads();
-    double top = 0;                                  // largest squared norm
-    for (int i = 0; i < K; i++) top = fmax(top, nrm[i]);
+    double top = largest(nrm, K);                    // largest squared norm
     const double unit = top > kTiny ? rcp_nr(sqrt_nr(top)) : 0.0;
     for (int e = tid; e < K * ldx; e += NT) X[e] = make_double2(X[e].x * unit, X[e].y * unit);
     __syncthreads();
@@ -192,9 +203,9 @@ __global__ void __launch_bounds__(kSmThreads, 1)
             const bool turn = g2 > kSkip || tt * tt < 1e-6f;
             const double tx = (double)(st * gx), ty = -(double)(st * gy);
             const double n2 = fma(tx, tx, fma(ty, ty, 1.0));
-            double co = (double)rsqrtf((float)n2);
-            co = fma(co, fma(-0.5 * n2 * co, co, 0.5), co);
-            co = fma(co, fma(-0.5 * n2 * co, co, 0.5), co);
+            double co = (double)rsqrtf((float)n2);   // 1e-7, cubed by one step of third order
+            const double er = fma(-n2 * co, co, 1.0);
+            co = fma(co * er, fma(er, 0.375, 0.5), co);
             const double sx = co * tx, sy = co * ty;
             if (have && turn) {    // u' = co u - s v, v' = co v + conj(s) u
               X[p * ldx + c0] = make_double2(fma(co, u.x, fma(-sx, v.x, sy * v.y)), fma(co, u.y, fma(-sx, v.y, -sy * v.x)));
@@ -218,8 +229,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     }
     __syncthreads();
     if (tid < K) {
-      top = 0;
-      for (int i = 0; i < K; i++) top = fmax(top, nrm[i]);
+      top = largest(nrm, K);
       vinv[tid] = nrm[tid] > fmax(floor2 * top, kTiny) ? rcp_nr(sqrt_nr(nrm[tid])) : 0.0;
     }
     __syncthreads();
@@ -254,10 +264,10 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     __syncthreads();
     // ---- descending order (ties by index), truncation as in k_select
     if (w == 0) {
-      const double mine = lane < K ? key[lane] : -1.0;
+      const long long mine = lane < K ? __double_as_longlong(key[lane]) : -1;   // not negative: ordered as integers
       int rank = 0;
       for (int i = 0; i < K; i++) {
-        const double o = key[i];
+        const long long o = __double_as_longlong(key[i]);
         rank += o > mine || (o == mine && i < lane) ? 1 : 0;
       }
       // NaN weights take no rank of their own: keep every slot a valid index
@@ -283,13 +293,19 @@ __global__ void __launch_bounds__(kSmThreads, 1)
       r = min(r, chi_max);
       const double kept = r == K ? W : wsum(lane < r ? k0 : 0.0);
       double* lam = P.lam_out[j];
-      if (lane < r) lam[lane] = kept > 0 ? sqrt(k0 / kept) : 0.0;
+      const bool plain = kept > 1e-280 && kept < 1e280 && W < 1e280;   // the fast routines' range
+      const double ik = plain ? rcp_nr(kept) : kept > 0 ? 1.0 / kept : 0.0;
+      if (lane < r) {
+        const double x = k0 * ik;
+        lam[lane] = plain && x > 1e-280 ? sqrt_nr(x) : sqrt(x);
+      }
       if (lane == 0) {
         double* res = P.res + 8 * (lev - 1);
-        res[0] = r; res[1] = W > 0 ? fmin(kept / W, 1.0) : 1.0; res[2] = W; res[3] = kept; res[4] = rc;
+        res[0] = r; res[1] = r == K || !(W > 0) ? 1.0 : fmin(plain ? kept * rcp_nr(W) : kept / W, 1.0); res[2] = W;
+        res[3] = kept; res[4] = rc;
         res[5] = sweep >= max_sweeps ? 1.0 : 0.0;
         r_s = r;
-        head[0] = kept > 0 ? 1.0 / sqrt(kept) : 0.0;
+        head[0] = plain ? rcp_nr(sqrt_nr(kept)) : kept > 0 ? 1.0 / sqrt(kept) : 0.0;
       }
     }
     __syncthreads();
@@ -326,8 +342,7 @@ size_t small_smem(int m, int n) {
 // shared memory.  Batched kernels / this kernel, whole calls: 10 FP64 clusters
 // of 4 sites at chi 8 4.8 / 4.0 ms; a run of 100 qubits at chi 256 (most of
 // its bonds narrow) 16.1 ms without, 13.5 with the limit at 8, 10.9 at 16; 12
-// exact FP64 qubits 3.4 / 2.2; one 16 x 16 split, the worst case, 0.24 / 0.27
-// in the kernels and 0.88 / 0.91 for the call.  Wider ones lose: an FP64
+// exact FP64 qubits 3.4 / 2.2; one 16 x 16 split 0.24 / 0.20 in the kernels.  Wider ones lose: an FP64
 // kernel of the same scheme took 3.4 ms in place of 1.7 at width 30.
 bool small_fits(int m, int n) { return n <= kSmMaxN && small_smem(m, n) <= kSmSmem; }
 
