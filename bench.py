@@ -1293,8 +1293,8 @@ def main():
                                  "randomized truncated SVD of the target design (sketch width l = r + 8, "
                                  "q = 0, CholeskyQR2, write-back; the l^3 small-SVD term excluded)"},
         "executed": {"tflops": tflops * world, "tc_frac": tflops * world / tc_peak,
-                     "definition": "algorithmic flops of the kernels this implementation runs (Gram, "
-                                   "Jacobi tile products, inner rotations, projections, merge, U)"},
+                     "definition": "algorithmic flops of the kernels this implementation runs (bidiagonalisation, "
+                                   "divide and conquer, back-transformation, projections, merge, U)"},
         "tc_peak": tc_peak, "tc_peak_source": mp["tf32_source"],
     }
     gpu_launches = int(sum(v["launches"] for v in counts.values()))
