@@ -204,7 +204,9 @@ int step(ctebd_mps* mps, const ctebd_cluster* c, int n, const double* const* U, 
 /* Eq. 5: product of all per-split fidelities so far (FP64). */
 int fidelity(const ctebd_mps* mps, double* F);
 
-/* <bits|psi>: bits has n_qubits entries in {0,1}, qubit 0 first. */
+/* <bits|psi>: bits has n_qubits entries in {0,1}, qubit 0 first.  Several
+   threads may ask one handle at once (calls take turns).
+   Errors: ARG, CUDA, OOM, TIMEOUT. */
 int amplitude(const ctebd_mps* mps, const uint8_t* bits, double* re, double* im);
 
 /* Current bond dimensions, n_qubits+1 entries. */

@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -559,6 +560,7 @@ struct ctebd_mps {
   size_t h_res_cap = 0;          // in problems
   std::map<int, Work> pending;
   Prof prof;
+  std::mutex read_lock;          // amplitude reads a const state, but through the staging block and dir_scr
 };
 
 // Stream-ordered memory from the handle's pool, which keeps up to kPoolKeep
@@ -2327,6 +2329,9 @@ extern "C" int amplitude(const ctebd_mps* mc, const uint8_t* bits, double* re, d
     fl += 8.0 * m->chi[q] * m->chi[q + 1];
   }
   const size_t bytes = amp_scratch_bytes(cmax);
+  // Threads may read one state side by side.  Descriptors, scratch, result and wait flag are the handle's, so one
+  // call at a time; all of them run on the handle's one stream anyway.
+  std::lock_guard<std::mutex> lock(m->read_lock);
   TRY(ensure_dir_scratch(m, bytes));
   TRY(ensure_tc_err(m));
   double2* out = reinterpret_cast<double2*>(m->dir_scr + bytes) - 1;
