@@ -31,8 +31,10 @@ static int fail(int code, const std::string& msg) {
 #define CUDA_TRY(call)                                                                   \
   do {                                                                                  \
     cudaError_t e_ = (call);                                                            \
-    if (e_ != cudaSuccess)                                                              \
+    if (e_ != cudaSuccess) {                                                            \
+      cudaGetLastError(); /* reported here, not again by the next call */               \
       return fail(CTEBD_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_));  \
+    }                                                                                   \
   } while (0)
 #define TRY(call)              \
   do {                         \
@@ -1560,11 +1562,7 @@ template <typename R>
 static int level_direct(ctebd_mps* m, std::vector<Work>& ws, const Level& L, const std::vector<int>& sel) {
   if (sel.empty()) return CTEBD_OK;
   // classes of similar width, one bidiagonalisation launch each
-  auto bucket = [&](int a) {
-    int b = 64;
-    while (b < L.nn[a]) b <<= 1;
-    return b;
-  };
+  auto bucket = [&](int a) { return dir_class(L.nn[a]); };
   std::vector<int> order(sel);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return bucket(x) > bucket(y); });
   const int na = (int)order.size();
@@ -1776,11 +1774,15 @@ static int level_sketch(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
 }
 
 // Full splits take the direct solver; the Jacobi solver keeps sketched splits,
-// runs with a low sweep cap (kDirectMinCap), and the policy that forces every
-// product onto the tensor cores.  4096 is the widest split of the ABI.
+// runs with a low sweep cap (kDirectMinCap), the policy that forces every
+// product onto the tensor cores, and matrices of more rows than the direct
+// solver's scratch takes (wide clusters of eight or nine qubits).  4096 is the
+// widest split of the ABI.
 constexpr int kDirectMaxWidth = 4096;
-static bool use_direct(int n) {
-  return g_max_sweeps >= kDirectMinCap && g_tc_mode != 2 && n <= kDirectMaxWidth;
+static bool direct_allowed() { return g_max_sweeps >= kDirectMinCap && g_tc_mode != 2; }
+static bool use_direct(const ctebd_mps* m, int rows, int n) {
+  return direct_allowed() && n <= kDirectMaxWidth &&
+         rows <= (m->fp64 ? dir_max_rows<double>(n, m->n_sm) : dir_max_rows<float>(n, m->n_sm));
 }
 
 // pass 1 (+ FP32 pass 2) for a selection: Gram of Z, eigen-solve, V, weights, select
@@ -1788,7 +1790,7 @@ static int level_solve(ctebd_mps* m, std::vector<Work>& ws, Level& L, const std:
   if (all.empty()) return CTEBD_OK;
   const bool f64 = m->fp64;
   std::vector<int> sel, direct;
-  for (int a : all) (!L.sk[a] && use_direct(L.nn[a]) ? direct : sel).push_back(a);
+  for (int a : all) (!L.sk[a] && use_direct(m, L.mm[a], L.nn[a]) ? direct : sel).push_back(a);
   if (!direct.empty()) {
     TRY(f64 ? level_direct<double>(m, ws, L, direct) : level_direct<float>(m, ws, L, direct));
     TRY(level_project_select(m, ws, L, direct));
@@ -1928,7 +1930,7 @@ static int rank_bound(const ctebd_mps* m, const Work& w, int j) {
   return (int)std::min({(long long)m->cfg.chi_max, (long long)w.chiL << j, (long long)w.chiR << (w.k - j)});
 }
 static bool use_small(const ctebd_mps* m, const Work& w, size_t& smem) {
-  if (!use_direct(1) || w.k > 12) return false;   // SmallProb holds 12 sites
+  if (!direct_allowed() || w.k > 12) return false;   // SmallProb holds 12 sites
   if (m->cfg.sketch_oversample > 0 && !m->fp64)
     for (int j = 0; j < w.k - 1; j++)
       if (w.hint[j] > 0) return false;          // a sketched split was asked for

@@ -84,6 +84,9 @@ struct DirProb {
 int dir_depth(int n);
 size_t dir_scratch_doubles(int n);
 void dir_carve(DirProb& q, double* p);
+int dir_class(int n);                       // launch class of a width: the widest of its members
+template <typename R>
+long long dir_max_rows(int n, int n_sm);    // the most rows that the class of width n takes
 // Golub-Kahan step of a class of problems (largest m and n of the class);
 // exchange scratch of dir_xchg_bytes (16-byte aligned), and a flag that a
 // bounded wait sets when it runs out
