@@ -321,6 +321,7 @@ struct Staging {
   unsigned char* h = nullptr;
   unsigned char* d = nullptr;
   size_t cap = 0, off = 0;
+  bool busy = false;               // something may still be on its way to the device
   cudaStream_t s = nullptr;
   std::vector<std::pair<unsigned char*, unsigned char*>> full;   // outgrown blocks, in use until reset
   unsigned char *first_h = nullptr, *first_d = nullptr;
@@ -349,14 +350,22 @@ struct Staging {
     if (first_d) cudaFree(first_d);
     h = d = first_h = first_d = nullptr;
   }
+  // At the start of a call: one that returned an error may have left copies behind.
+  int settle() {
+    if (busy) CUDA_TRY(cudaStreamSynchronize(s));
+    reset();
+    return CTEBD_OK;
+  }
   // Callers reset only after a stream synchronisation.
   void reset() {
     off = 0;
+    busy = false;
     if (!full.empty()) drop_full();
   }
   // room for `bytes` at h + *at and d + *at
   int room(size_t bytes, size_t* at) {
     const size_t need = (bytes + 255) & ~size_t(255);
+    busy = true;
     if (off + need > cap) {
       if (need > kMax) {
         CUDA_TRY(cudaStreamSynchronize(s));
@@ -2180,13 +2189,14 @@ extern "C" int step(ctebd_mps* m, const ctebd_cluster* c, int n, const double* c
   }
   m->splitlog.clear();
   m->splitlog2.clear();
-  m->stage.reset();
+  TRY(m->stage.settle());
   TRY(carve_work(m, ws));
   std::vector<const double*> Us(U, U + n);
   TRY(merge_apply(m, ws, Us));
   std::vector<std::vector<double>> fs;
   TRY(split_levels(m, ws, fs, ++m->nstep));
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   TRY(check_tc_flag(m));
   if (f_out) {
     size_t o = 0;
@@ -2200,8 +2210,8 @@ extern "C" int apply_cluster(ctebd_mps* m, const ctebd_cluster* c, const double*
   Work w;
   TRY(make_work(m, c, w));
   if (m->pending.count(c->q0)) return fail(CTEBD_ERR_STATE, "apply_cluster: cluster already pending");
-  m->stage.reset();
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   TRY(alloc_owned(m, w));
   std::vector<Work> ws{w};
   std::vector<const double*> Us{U};
@@ -2209,6 +2219,7 @@ extern "C" int apply_cluster(ctebd_mps* m, const ctebd_cluster* c, const double*
   if (rc) { free_owned(m, ws[0]); return rc; }
   m->pending[c->q0] = ws[0];
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   return CTEBD_OK;
 }
 
@@ -2216,24 +2227,25 @@ extern "C" int truncate_split(ctebd_mps* m, const ctebd_cluster* c, double* f_ou
   if (!m || !c) return fail(CTEBD_ERR_ARG, "truncate_split: null argument");
   auto it = m->pending.find(c->q0);
   if (it == m->pending.end() || it->second.k != c->k) return fail(CTEBD_ERR_STATE, "truncate_split: no pending apply_cluster for this cluster");
+  TRY(m->stage.settle());
   std::vector<Work> ws{it->second};
   m->pending.erase(it);
   m->splitlog.clear();
-  m->stage.reset();
   std::vector<std::vector<double>> fs;
   m->splitlog2.clear();
   int rc = split_levels(m, ws, fs, ++m->nstep);
   free_owned(m, ws[0]);
   if (rc) return rc;
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   if (f_out) for (size_t i = 0; i < fs[0].size(); i++) f_out[i] = fs[0][i];
   return CTEBD_OK;
 }
 
 extern "C" int apply_1q(ctebd_mps* m, int q, const double* u) {
   if (!m || !u || q < 0 || q >= m->n) return fail(CTEBD_ERR_ARG, "apply_1q: bad args");
-  m->stage.reset();
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   void* s = m->site[q];
   const int cl = m->chi[q], cr = m->chi[q + 1];
   Staging::Set set;
@@ -2338,7 +2350,7 @@ extern "C" int amplitude(const ctebd_mps* mc, const uint8_t* bits, double* re, d
   TRY(ensure_tc_err(m));
   double2* out = reinterpret_cast<double2*>(m->dir_scr + bytes) - 1;
   const AmpSite* ds;
-  m->stage.reset();   // every call has waited for the stream before it returned
+  TRY(m->stage.settle());
   TRY(m->stage.push(sites.data(), sites.size(), &ds));
   const int ctas = amp_ctas(cmax, m->n_sm), mid = m->chi[m->n / 2];
   int* h_flag = reinterpret_cast<int*>(m->h_res + 16 * m->h_res_cap);
@@ -2352,6 +2364,7 @@ extern "C" int amplitude(const ctebd_mps* mc, const uint8_t* bits, double* re, d
   CUDA_TRY(cudaMemcpyAsync(m->h_res, out, sizeof(double2), cudaMemcpyDeviceToHost, m->stream));
   CUDA_TRY(cudaMemcpyAsync(h_flag, m->tc_err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   if (*h_flag) return check_tc_flag(m);
   *re = m->h_res[0];
   *im = m->h_res[1];
@@ -2466,7 +2479,7 @@ extern "C" int mps_load_device(ctebd_mps* m, const int* chi, const void* const* 
   }
   for (int b = 0; b <= m->n; b++) TRY(add(m->lam[b], lams[b], sizeof(double) * chi[b], cudaMemcpyDefault));
   if (!cp.empty()) {
-    m->stage.reset();   // every call has waited for the stream before it returned
+    TRY(m->stage.settle());
     const CopyProb* dc;
     TRY(m->stage.push(cp.data(), cp.size(), &dc));
     CUDA_TRY(launch_copy_batch(dc, (int)cp.size(), (long long)largest, m->stream));
@@ -2474,6 +2487,7 @@ extern "C" int mps_load_device(ctebd_mps* m, const int* chi, const void* const* 
   m->chi.assign(chi, chi + m->n + 1);
   m->logF = 0;
   CUDA_TRY(cudaStreamSynchronize(m->stream));
+  m->stage.reset();
   return CTEBD_OK;
 }
 
