@@ -1784,9 +1784,9 @@ static int level_sketch(ctebd_mps* m, std::vector<Work>& ws, const Level& L, con
 
 // Full splits take the direct solver; the Jacobi solver keeps sketched splits,
 // runs with a low sweep cap (kDirectMinCap), the policy that forces every
-// product onto the tensor cores, and matrices of more rows than the direct
-// solver's scratch takes (wide clusters of eight or nine qubits).  4096 is the
-// widest split of the ABI.
+// product onto the tensor cores, matrices of more rows than the direct solver's
+// scratch takes (wide clusters of eight or nine qubits), and tall ones where it
+// is the faster one (gram_is_faster).  4096 is the widest split of the ABI.
 constexpr int kDirectMaxWidth = 4096;
 static bool direct_allowed() { return g_max_sweeps >= kDirectMinCap && g_tc_mode != 2; }
 static bool use_direct(const ctebd_mps* m, int rows, int n) {
@@ -1794,12 +1794,51 @@ static bool use_direct(const ctebd_mps* m, int rows, int n) {
          rows <= (m->fp64 ? dir_max_rows<double>(n, m->n_sm) : dir_max_rows<float>(n, m->n_sm));
 }
 
+// Tall matrices (m >= 8 n, clusters of five and more qubits).  Reading the
+// matrix once for its Gram matrix and solving that costs less than passing over
+// its trailing part twice per column, one problem after another, when the rows
+// of a level's problems do not fit the chip's shared memory side by side.  The
+// rule compares estimates in microseconds per level, for c problems:
+//   direct  c n (2 + 2e-6 m n),  3e-6 beyond 72 MB (L2);  FP64 c n (3 + 3.2e-5 m n);
+//           2.4 times the second term at 65 to 128 columns
+//   Gram    45 n + c (3.5e-6 n^3 + 0.55e-6 m n^2);  FP64 160 n + c (3e-4 n^3 + 1.2e-5 m n^2)
+// fitted to both sides of 124 shapes (16 to 2048 columns, 512 to 65536 rows, 1
+// to 16 problems, flat spectra).  Direct / Gram, ms of solver time per level:
+//   FP32  8192 x 512: 1 problem 6.9 / 27, 4: 24 / 29, 8: 47 / 36
+//         32768 x 512: 1: 28 / 27, 4: 107 / 38;  8192 x 1024: 4: 75 / 100
+//         16384 x 1024: 1: 52 / 61, 4: 201 / 92;  65536 x 1024: 1: 244 / 76
+//         8192 x 2048: 2: 177 / 228;  16384 x 2048: 1: 217 / 199, 2: 430 / 289
+//   FP64  4096 x 128: 4: 26 / 21, 16: 100 / 38;  8192 x 512: 4: 269 / 363
+// The rule takes the faster side of all but six of them, there at most 1.27
+// times the other.  At m = 4 n and below the direct solver is the faster one.
+static bool gram_is_faster(const ctebd_mps* m, const Level& L, const std::vector<int>& tall) {
+  const bool f64 = m->fp64;
+  double all = 0, direct = 0, gram = 0, widest = 0;
+  for (int a : tall) {
+    const double mm = L.mm[a], n = L.nn[a], bytes = mm * n * (double)m->esz;
+    const double pass = (f64 ? 3.2e-5 : bytes <= 72e6 ? 2e-6 : 3e-6) * (n > 64 && n <= 128 ? 2.4 : 1.0);
+    direct += n * ((f64 ? 3 : 2) + pass * mm * n);
+    gram += f64 ? 3e-4 * n * n * n + 1.2e-5 * mm * n * n : 3.5e-6 * n * n * n + 0.55e-6 * mm * n * n;
+    all += bytes;
+    widest = std::max(widest, n);
+  }
+  return all > m->n_sm * 226e3 && direct > gram + (f64 ? 160 : 45) * widest;
+}
+
 // pass 1 (+ FP32 pass 2) for a selection: Gram of Z, eigen-solve, V, weights, select
 static int level_solve(ctebd_mps* m, std::vector<Work>& ws, Level& L, const std::vector<int>& all) {
   if (all.empty()) return CTEBD_OK;
   const bool f64 = m->fp64;
   std::vector<int> sel, direct;
-  for (int a : all) (!L.sk[a] && use_direct(m, L.mm[a], L.nn[a]) ? direct : sel).push_back(a);
+  std::map<int, std::vector<int>> tall;      // by launch class
+  for (int a : all)
+    if (L.sk[a] || !use_direct(m, L.mm[a], L.nn[a])) sel.push_back(a);
+    else if (L.mm[a] < 8 * L.nn[a]) direct.push_back(a);
+    else tall[dir_class(L.nn[a])].push_back(a);
+  for (const auto& t : tall) {
+    std::vector<int>& to = gram_is_faster(m, L, t.second) ? sel : direct;
+    to.insert(to.end(), t.second.begin(), t.second.end());
+  }
   if (!direct.empty()) {
     TRY(f64 ? level_direct<double>(m, ws, L, direct) : level_direct<float>(m, ws, L, direct));
     TRY(level_project_select(m, ws, L, direct));
