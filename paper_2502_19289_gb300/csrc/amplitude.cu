@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kAmpThreads, 1)
       for (int j = tid; need && j < cur.outs; j += kAmpThreads) {
         const unsigned char* ad[1] = {buf + (size_t)j * SB};
         double2 v[1];
-        if (!poll(ad, seq, v, err)) bad = 1;
+        if (!poll(ad, seq, v, err, kWaitAmplitude)) bad = 1;
         vs[j] = v[0];
       }
     } else {

@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(NT, 1) k_eig_apply_tc(const EigProb* __restric
   __syncthreads();
   t5::fence_after();
   if (warp == 0) t5::tmem_dealloc(tmem, TMEM_COLS);
-  if (failed && t == 0) atomicExch(err, 1);
+  if (failed && t == 0) atomicCAS(err, kWaitNone, kWaitTensor);
 }
 
 }  // namespace

@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "waits.h"
+
 namespace ctebd {
 
 // ---- exchange between the CTAs of a group ------------------------------------
@@ -9,7 +11,8 @@ namespace ctebd {
 // sequence number, and the reader polls the value itself: one trip through L2
 // instead of data, fence, flag and data again.  A slot's value is valid when
 // its sequence number is the step's; the slots are zeroed before the launch
-// and numbers start at 1.  Polls are bounded: one that runs out sets *err.
+// and numbers start at 1.  Polls are bounded: one that runs out sets *err to the
+// caller's code (waits.h); the first one's stays.
 constexpr int kSpinLimit = 1 << 21;
 
 __device__ __forceinline__ void st128(void* p, unsigned long long lo, unsigned long long hi) {
@@ -55,7 +58,8 @@ template <> struct Slot<double2> {
 // them from the first poll on: waiting for one and then reading the others
 // costs another trip, 28.1 -> 29.5 ms for two 2048-wide problems.)
 template <int N, typename CT>
-__device__ __forceinline__ bool poll(const unsigned char* const (&p)[N], unsigned seq, CT (&v)[N], int* err) {
+__device__ __forceinline__ bool poll(const unsigned char* const (&p)[N], unsigned seq, CT (&v)[N], int* err,
+                                     int code) {
   bool have[N];
 #pragma unroll
   for (int i = 0; i < N; i++) { have[i] = p[i] == nullptr; v[i] = CT{0, 0}; }
@@ -69,7 +73,7 @@ __device__ __forceinline__ bool poll(const unsigned char* const (&p)[N], unsigne
     if (all) return true;
     if ((it & 1023) == 1023 && *(volatile int*)err) break;
   }
-  atomicExch(err, 1);
+  atomicCAS(err, kWaitNone, code);
   return false;
 }
 

@@ -551,7 +551,7 @@ struct ctebd_mps {
                                    // largest last-sweep moved weight (relative to the trace)
   uint64_t nstep = 0;
   float* mlp = nullptr;            // rank predictor parameters (device)
-  int* tc_err = nullptr;           // tensor-core completion-wait timeout flag (device)
+  int* tc_err = nullptr;           // which bounded wait ran out (waits.h; device)
   double* eig_scr = nullptr;       // eigen-solve counters and pair flags (high-water)
   size_t eig_scr_cap = 0;          // in doubles
   unsigned char* pack_scr = nullptr;   // packed tensor-core GEMM operands (high-water)
@@ -764,7 +764,7 @@ static int ensure_pack_scratch(ctebd_mps* m, size_t n) {
   return CTEBD_OK;
 }
 
-// the device flag that a tensor-core kernel sets when a bounded wait expires
+// the device flag that a kernel sets when a bounded wait expires
 static int ensure_tc_err(ctebd_mps* m) {
   if (m->tc_err) return CTEBD_OK;
   CUDA_TRY(cudaMalloc(&m->tc_err, sizeof(int)));
@@ -2203,14 +2203,14 @@ static int make_work(ctebd_mps* m, const ctebd_cluster* c, Work& w) {
   return CTEBD_OK;
 }
 
-// a tensor-core completion wait that ran out sets the flag; report and clear it
+// a bounded wait that ran out sets the flag (waits.h); report and clear it
 static int check_tc_flag(ctebd_mps* m) {
   if (!m->tc_err) return CTEBD_OK;
   int h = 0;
   CUDA_TRY(cudaMemcpy(&h, m->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (!h) return CTEBD_OK;
   CUDA_TRY(cudaMemset(m->tc_err, 0, sizeof(int)));
-  return fail(CTEBD_ERR_TIMEOUT, "a tensor-core completion wait timed out");
+  return fail(CTEBD_ERR_TIMEOUT, std::string(wait_name(h)) + " timed out");
 }
 
 extern "C" int step(ctebd_mps* m, const ctebd_cluster* c, int n, const double* const* U, double* f_out) {

@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <string>
 
+#include "waits.h"
+
 namespace ctebd {
 
 // One complex GEMM of a grouped launch, interleaved complex of real type R:

@@ -1,7 +1,9 @@
 // Host program of test_gpu_numeric.py: evaluates the scalar routines of
 // numeric.cuh and pair.cuh on numbers from standard input (FP64, binary) and
-// writes the results as FP64 numbers (high and low part of each).
+// writes the results as FP64 numbers (high and low part of each), or lets a
+// bounded wait run out.
 //   numeric_probe FUNCTION COUNT     sqrt32 rcp32 sqrt64 rcp64 pair_sqrt pair_rcp
+//   numeric_probe wait 0             one poll of a slot that nothing fills
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -9,6 +11,7 @@
 #include <cstring>
 #include <vector>
 
+#include "exchange.cuh"
 #include "numeric.cuh"
 #include "pair.cuh"
 
@@ -34,12 +37,31 @@ __global__ void k_eval(int fn, const double* x, double* out, int n) {
   out[2 * i + 1] = l;
 }
 
+__global__ void k_wait(const unsigned char* slot, int* err, int* ok) {
+  const unsigned char* ad[1] = {slot};
+  float2 v[1];
+  *ok = poll(ad, 1u, v, err, kWaitSplit) ? 1 : 0;
+}
+
 static void check(cudaError_t e) {
   if (e != cudaSuccess) { std::fprintf(stderr, "%s\n", cudaGetErrorString(e)); std::exit(1); }
 }
 
 int main(int argc, char** argv) {
   if (argc < 3) return 2;
+  if (!std::strcmp(argv[1], "wait")) {
+    unsigned char* slot;
+    int *w, h[2];
+    check(cudaMalloc(&slot, 64));
+    check(cudaMalloc(&w, sizeof(h)));
+    check(cudaMemset(slot, 0, 64));
+    check(cudaMemset(w, 0, sizeof(h)));
+    k_wait<<<1, 1>>>(slot, w, w + 1);
+    check(cudaDeviceSynchronize());
+    check(cudaMemcpy(h, w, sizeof(h), cudaMemcpyDeviceToHost));
+    std::printf("%d %d %s\n", h[0], h[1], wait_name(h[0]));
+    return 0;
+  }
   const char* names[] = {"sqrt32", "rcp32", "sqrt64", "rcp64", "pair_sqrt", "pair_rcp"};
   int fn = -1;
   for (int i = 0; i < 6; i++)

@@ -3,7 +3,10 @@ reciprocal by Newton's iteration, in FP32, FP64 and pairs of FP32 numbers)
 against extended precision, over the ranges that their comments state.
 
 Bounds (derived there): half an ulp and a fiftieth of it, 1.02 x 2^-24 and
-1.02 x 2^-53 relative, and 2^-44 for pairs."""
+1.02 x 2^-53 relative, and 2^-44 for pairs.
+
+Also here: a bounded wait of exchange.cuh on a slot that nothing fills ends, and
+says which kernel waited."""
 import os
 import subprocess
 
@@ -54,3 +57,8 @@ def test_scalar_routine(probe, fn):
     err = np.abs(got - want) / want
     print(f"{fn}: largest relative error 2^{float(np.log2(err.max())):.2f}")
     assert err.max() <= bound
+
+
+def test_wait_that_runs_out_names_its_kernel(probe):
+    out = subprocess.run([probe, "wait", "0"], check=True, capture_output=True, text=True, timeout=60).stdout
+    assert out.strip() == "2 0 an exchange of the direct split"
