@@ -574,10 +574,45 @@ struct ctebd_mps {
   std::mutex read_lock;          // amplitude reads a const state, but through the staging block and dir_scr
 };
 
-// Stream-ordered memory from the handle's pool, which keeps up to kPoolKeep
-// bytes between calls: the device's default pool gives everything back at each
-// synchronisation (95 us for an allocation and its release).
+// Stream-ordered memory from the handle's pool, which keeps some bytes between
+// calls: the device's default pool gives everything back at each
+// synchronisation (95 us for an allocation and its release).  All handles of the
+// process together keep at most kPoolKeep bytes, in equal shares: the share of a
+// handle is kPoolKeep over the number of handles rounded up to a power of two
+// (so that the others are told only when that changes, and on the way down only
+// at a quarter of it), and what a pool holds beyond a smaller share is given back.
 constexpr uint64_t kPoolKeep = (uint64_t)1 << 30;
+static std::mutex g_pools_lock;
+static std::vector<cudaMemPool_t> g_pools;
+static size_t g_pool_shares = 1;
+
+static cudaError_t pool_share(cudaMemPool_t p) {
+  uint64_t keep = kPoolKeep / g_pool_shares;
+  const cudaError_t e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+  return e != cudaSuccess ? e : cudaMemPoolTrimTo(p, keep);
+}
+static cudaError_t pool_open(cudaMemPool_t* p, const cudaMemPoolProps& props) {
+  cudaError_t e = cudaMemPoolCreate(p, &props);
+  if (e != cudaSuccess) { *p = nullptr; return e; }
+  std::lock_guard<std::mutex> lock(g_pools_lock);
+  g_pools.push_back(*p);
+  if (g_pools.size() <= g_pool_shares) return pool_share(*p);
+  g_pool_shares *= 2;
+  for (cudaMemPool_t q : g_pools)
+    if (cudaError_t r = pool_share(q)) e = r;
+  return e;
+}
+static void pool_close(cudaMemPool_t p) {
+  {
+    std::lock_guard<std::mutex> lock(g_pools_lock);
+    g_pools.erase(std::find(g_pools.begin(), g_pools.end(), p));
+    if (g_pool_shares > 1 && g_pools.size() <= g_pool_shares / 4) {
+      g_pool_shares /= 2;
+      for (cudaMemPool_t q : g_pools) pool_share(q);
+    }
+  }
+  cudaMemPoolDestroy(p);
+}
 template <typename T> static cudaError_t pool_alloc(ctebd_mps* m, T** p, size_t bytes) {
   return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, m->pool, m->stream);
 }
@@ -650,9 +685,8 @@ extern "C" int mps_create(const ctebd_config* cfg, void* cuda_stream, ctebd_mps*
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = dev;
-  uint64_t keep = kPoolKeep;
-  if (cudaMemPoolCreate(&m->pool, &props) != cudaSuccess ||
-      cudaMemPoolSetAttribute(m->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+  if (pool_open(&m->pool, props) != cudaSuccess) {
+    cudaGetLastError();
     mps_destroy(m);
     return fail(CTEBD_ERR_CUDA, "mps_create: memory pool");
   }
@@ -701,7 +735,7 @@ extern "C" int mps_destroy(ctebd_mps* m) {
   for (void* p : m->site) if (p && !in_site_block(m, p)) cudaFreeAsync(p, m->stream);
   if (m->site_block) cudaFreeAsync(m->site_block, m->stream);
   if (m->stream) cudaStreamSynchronize(m->stream);
-  if (m->pool) cudaMemPoolDestroy(m->pool);
+  if (m->pool) pool_close(m->pool);
   if (m->lam_block) cudaFree(m->lam_block);
   if (m->arena) cudaFree(m->arena);
   if (m->mlp) cudaFree(m->mlp);
