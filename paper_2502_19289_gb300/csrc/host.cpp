@@ -866,7 +866,7 @@ static int launch_gemm_group(ctebd_mps* m, const std::vector<GemmProb>& probs, i
     return CTEBD_OK;
   }
   std::vector<long long> off(probs.size() + 1, 0);
-  const int tm = gemm_tile(probs.data(), (int)probs.size(), m->fp64);
+  const int tm = gemm_tile(probs.data(), (int)probs.size(), m->fp64, m->n_sm);
   for (size_t i = 0; i < probs.size(); i++) off[i + 1] = off[i] + gemm_tiles(probs[i], tm);
   Staging::Set set;
   const size_t ip = set.add(probs.data(), probs.size()), io = set.add(off.data(), off.size());

@@ -202,7 +202,7 @@ template <typename R>
 cudaError_t launch_gemm(const GemmProb* d_probs, const long long* d_tile_off, int n_probs,
                         long long total_tiles, int tm, cudaStream_t s);
 // host: the tile (16 tm x 16 tm) for a group of problems, and a problem's tiles in the grid
-int gemm_tile(const GemmProb* probs, int n, bool fp64);
+int gemm_tile(const GemmProb* probs, int n, bool fp64, int n_sm);
 long long gemm_tiles(const GemmProb& p, int tm);
 
 template <typename R>

@@ -143,7 +143,7 @@ long long gemm_tiles(const GemmProb& p, int tm) {
   return (long long)((p.M + bm - 1) / bm) * ((p.N + bm - 1) / bm) * p.batch;
 }
 
-// Rule: the tile whose waves over 152 SMs cost least, a wave of 16 TM costing
+// Rule: the tile whose waves over the SMs cost least, a wave of 16 TM costing
 // TM^2 (FP32: times 1.3 and 2 for the two smaller ones, which read shared
 // memory more often per product).  Products of the splits are small next to
 // the chip -- FP64 runs at 2 lanes a clock and SM, so every idle SM counts.
@@ -152,14 +152,13 @@ long long gemm_tiles(const GemmProb& p, int tm) {
 // FP64 30-wide 0.074 + 0.143 / 0.027 + 0.047 / 0.019 + 0.023; sixteen FP32
 // 48-wide 0.065 + 0.092 / 0.051 + 0.058 / 0.038 + 0.058; eight FP32 200-wide
 // 0.087 + 0.147 / 0.074 + 0.138 / 0.092 + 0.162.
-int gemm_tile(const GemmProb* probs, int n, bool fp64) {
-  constexpr long long kSms = 152;
+int gemm_tile(const GemmProb* probs, int n, bool fp64, int n_sm) {
   int best = 4;
   double cost = 0;
   for (int tm = 4; tm >= 1; tm >>= 1) {
     long long tiles = 0;
     for (int i = 0; i < n; i++) tiles += gemm_tiles(probs[i], tm);
-    const double c = (double)((tiles + kSms - 1) / kSms) * tm * tm * (fp64 || tm == 4 ? 1.0 : tm == 2 ? 1.3 : 2.0);
+    const double c = (double)((tiles + n_sm - 1) / n_sm) * tm * tm * (fp64 || tm == 4 ? 1.0 : tm == 2 ? 1.3 : 2.0);
     if (tm == 4 || c < cost) { best = tm; cost = c; }
   }
   return best;

@@ -89,6 +89,7 @@ struct NaDesc {
   unsigned char* base;
   size_t off = 0;
   cudaStream_t s;
+  int n_sm;
   template <typename T>
   int put(const T* src, size_t count, const T** dst) {
     const size_t bytes = sizeof(T) * count, need = al256(bytes);
@@ -105,7 +106,7 @@ static int na_gemm(NaDesc& d, const GemmProb& p) {
     GemmProb p;
     long long off[2];
   } h = {p, {0, 0}};
-  const int tm = gemm_tile(&p, 1, false);
+  const int tm = gemm_tile(&p, 1, false, d.n_sm);
   h.off[1] = gemm_tiles(p, tm);
   const One* dp;
   if (int rc = d.put(&h, 1, &dp)) return rc;
@@ -163,10 +164,7 @@ static int na_eig(NaDesc& d, unsigned char* S, void* acc, int npad, double floor
 // path's), in V: reflectors in the Gram area, eigenvectors in the refinement
 // accumulator, everything else in the area of the projection that follows.
 static int na_direct(NaDesc& d, unsigned char* S, int m, int n, int npad, const double* lamL, int* flag) {
-  int dev = 0, n_sm = 0;
-  NA_CUDA(cudaGetDevice(&dev));
-  NA_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  const size_t xchg = al256(dir_xchg_bytes<float>(m, n, 1, n_sm));
+  const size_t xchg = al256(dir_xchg_bytes<float>(m, n, 1, d.n_sm));
   if (xchg + dir_scratch_doubles(n) * sizeof(double) > NA_OFF_G - NA_OFF_RFULL)
     return na_fail(CTEBD_ERR_ARG, "split2_noalloc: internal: direct solver scratch");
   DirProb q{};
@@ -181,7 +179,7 @@ static int na_direct(NaDesc& d, unsigned char* S, int m, int n, int npad, const 
   if (int rc = d.put(&q, 1, &dq)) return rc;
   NA_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), d.s));
   int launches = 0;
-  NA_CUDA(launch_dir_bidiag<float>(dq, 1, m, n, S + NA_OFF_RFULL, flag, n_sm, d.s));
+  NA_CUDA(launch_dir_bidiag<float>(dq, 1, m, n, S + NA_OFF_RFULL, flag, d.n_sm, d.s));
   NA_CUDA(launch_dir_tridiag<float>(dq, 1, n, &launches, d.s));
   NA_CUDA(launch_dir_back<float>(dq, 1, n, d.s));
   return CTEBD_OK;
@@ -236,7 +234,10 @@ extern "C" int split2_noalloc(const void* theta, const double* lam_l, int chi_l,
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int m = 2 * chi_l, n = 2 * chi_r;
   const int npad = (n + 2 * NA_JB - 1) / (2 * NA_JB) * (2 * NA_JB);
-  NaDesc d{S + NA_OFF_DESC, 0, s};
+  int dev = 0, n_sm = 0;
+  NA_CUDA(cudaGetDevice(&dev));
+  NA_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  NaDesc d{S + NA_OFF_DESC, 0, s, n_sm};
   // Mbar: copy of theta viewed (chi_l * 2) x (2 * chi_r)
   NA_CUDA(cudaMemcpyAsync(S + NA_OFF_MBAR, theta, (size_t)m * n * NA_CPLX, cudaMemcpyDeviceToDevice, s));
   void* V = S + NA_OFF_V;
