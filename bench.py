@@ -51,6 +51,31 @@ APPLY_TRAFFIC = {
 }
 
 
+# DRAM traffic of the bidiagonalisation (k_bidiag) per algorithmic flop, from one
+# ncu capture of run_bidiag_traffic at n = 32: one level of a saturated chi =
+# 1024 iteration, the cluster sizes of the default workload.  Null once the
+# kernel's source changes.
+BIDIAG_TRAFFIC = {
+    "bytes_per_flop": (117199380992 + 189555739648) / 462066898261.3,
+    "source_sha256": "9bd3cec63e13aec51b5aa411346ad27f44b7b1e5a3782f34db7c6b38c6015a22",
+    "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the first k_bidiag launch of "
+               "'bench.py --workload bidiag-traffic --n 32' on a GB300 (2048 columns and 512, 2048, 2048, 4096 and "
+               "8192 rows; the launch keeps its rows in global memory): 117,199,380,992 + 189,555,739,648 B for "
+               "4.621e11 algorithmic flops, scaled to this launch's flops",
+}
+
+
+def bidiag_kernel_digest() -> str:
+    """sha256 of the bidiagonalisation kernel's source text (comment and body)
+    and of its launch plan."""
+    src = open(os.path.join(ROOT, "paper_2502_19289_gb300", "csrc", "svd_direct.cu")).read()
+    a = src.index("// One Golub-Kahan step per column k.")
+    b = src.index("\n}\n", src.index("k_bidiag(const DirProb*", a)) + 3
+    c = src.index("// Launch shape of a class of problems")
+    d = src.index("\n}\n", c) + 3
+    return hashlib.sha256((src[a:b] + src[c:d]).encode()).hexdigest()
+
+
 def apply_kernel_digest() -> str:
     """sha256 of the FP32 round-update kernel's source text (comment, tile
     constants and kernel body)."""
@@ -60,12 +85,15 @@ def apply_kernel_digest() -> str:
     return hashlib.sha256(src[a:b].encode()).hexdigest()
 
 
-def apply_traffic_per_launch(flops_per_launch: float):
-    """(bytes, note) for a round-update launch of the given algorithmic flops."""
-    t = APPLY_TRAFFIC
+def traffic_per_launch(kernel: str, flops_per_launch: float):
+    """(bytes, note) for a launch of the given algorithmic flops."""
+    known = {"eig_apply": (APPLY_TRAFFIC, apply_kernel_digest), "bidiag": (BIDIAG_TRAFFIC, bidiag_kernel_digest)}
+    if kernel not in known:
+        return None, "no capture of this kernel"
+    t, digest = known[kernel]
     if t["bytes_per_flop"] is None:
         return None, "no capture"
-    if t["source_sha256"] != apply_kernel_digest():
+    if t["source_sha256"] != digest():
         return None, "kernel changed since the capture"
     return t["bytes_per_flop"] * flops_per_launch, t["capture"]
 
@@ -343,7 +371,7 @@ def mps_overlap(torch, a_sites, b_sites):
 def run_compare(args):
     """The same iterations three ways from one state: the library's FP32 path
     (batched, tensor cores), the library's FP64 mode (same kernels and
-    batching in complex128 / FP64 Jacobi) and the plain FP64 GPU path
+    batching in complex128) and the plain FP64 GPU path
     (PlainFP64).  Workload: the chi_max = 1024 workload's circuit statistics on
     an n-qubit state saturated at chi; every arm runs `steps` iterations after
     one untimed warm-up iteration; device time of the updates with CUDA events.
@@ -444,8 +472,9 @@ def run_compare(args):
 
 def run_apply_traffic(args):
     """Small case for the dominant kernel's DRAM traffic per algorithmic flop:
-    one saturated chi = 1024 iteration on n qubits (host-generated state,
-    host-driven sweep rounds so that every launch is visible to a profiler).
+    one saturated chi = 1024 iteration on n qubits (host-generated state) by the
+    Jacobi solver (a sweep cap below the direct solver's, host-driven sweep
+    rounds so that every launch is visible to a profiler).
     Prints the eigenproblems of the first eigen-solve and the algorithmic flops
     of its first round update, in which every pair of column blocks rotates:
     one 64^3 complex product per V tile and two per upper G tile.  Captured as
@@ -467,15 +496,46 @@ def run_apply_traffic(args):
     mps = P.MPS(cfg)
     mps.load(chis, sites, lams)
     P.set_sweep_graphs(0)
+    P.set_max_sweeps(11)
     clusters, stop = P.cluster_partition(circ.gates, circ.n_gates, 0, mps.bond_dims(), cfg)
     Us = [P.cluster_unitary(circ.gates, circ.n_gates, cl) for cl in clusters]
-    mps.step(clusters, Us)
-    log = mps.split_log()
-    level1 = [row for row in log if int(row[2]) == int(row[0]) + int(row[1]) - 1]
-    h = [((int(row[9]) + 63) // 64 * 64) // 64 for row in level1]   # pairs of 32-wide blocks
+    widths = [2 * int(chis[cl.q0 + cl.k]) for cl in clusters]   # of the first splits
+    try:
+        mps.step(clusters, Us)
+    except P.CtebdError:   # a solve that needs more sweeps than the cap; the first round is what is captured
+        pass
+    h = [(n + 63) // 64 for n in widths]   # pairs of 32-wide blocks
     flops = sum(8.0 * 64 ** 3 * (2 * (x * (x + 1) // 2) + x * x) for x in h)
-    print(json.dumps({"problems": len(h), "widths": sorted(set(int(r[9]) for r in level1)),
+    print(json.dumps({"problems": len(h), "widths": sorted(set(widths)),
                       "first_round_flops": flops, "source_sha256": apply_kernel_digest()}))
+
+
+def run_bidiag_traffic(args):
+    """The same iteration by the direct solver: prints the splits of the first
+    level's widest launch class and the algorithmic flops of their
+    bidiagonalisation, 16 (m n k - (m + n) k^2 / 2 + k^3 / 3) with k = min(m, n).
+    Captured as
+
+        python bench.py --workload bidiag-traffic --n 32 &&
+        ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
+            --clock-control none -k regex:k_bidiag -c 1 --csv
+            python bench.py --workload bidiag-traffic --n 32"""
+    import paper_2502_19289_gb300 as P
+    import synth
+    n = args.n
+    w = synth.WORKLOADS[4]
+    cfg = P.make_config(n, 1024, w.cutoff, 24, 0, 4, P.FP32)
+    c = synth.random_structured(n, w.n_layers, p1=w.p1, p2=w.p2, one_q=w.one_q, two_q=w.two_q, seed=4000)
+    circ = P.Circuit(n, c.gates, c.params)
+    chis, sites, lams = synth.random_right_canonical(n, 1024, seed=4000, dtype=np.complex64)
+    mps = P.MPS(cfg)
+    mps.load(chis, sites, lams)
+    clusters, stop = P.cluster_partition(circ.gates, circ.n_gates, 0, mps.bond_dims(), cfg)
+    mps.step(clusters, [P.cluster_unitary(circ.gates, circ.n_gates, cl) for cl in clusters])
+    level1 = [(int(r[3]), int(r[4])) for r in mps.split_log() if int(r[2]) == int(r[0]) + int(r[1]) - 1]
+    wide = [(a, b) for a, b in level1 if 1024 < b <= 2048]
+    flops = sum(16.0 * (a * b * min(a, b) - (a + b) * min(a, b) ** 2 / 2 + min(a, b) ** 3 / 3) for a, b in wide)
+    print(json.dumps({"splits": wide, "flops": flops, "source_sha256": bidiag_kernel_digest()}))
 
 
 def run_cfg5(args):
@@ -570,10 +630,7 @@ def run_latency(args):
     of the library's kernels in a second, identical run with per-launch CUDA
     events.  Their ratio is the fraction of the step the GPU is busy; the rest
     is host work, launch gaps and the per-level reads, the most that capturing
-    a whole step into one graph could remove.  The first run takes the
-    default sweep-loop policy (device-side graphs for batches at least 16
-    blocks wide); two more drive every eigen-solve's sweep loop from the host,
-    then every one from a device-side graph."""
+    a whole step into one graph could remove."""
     import torch
 
     import paper_2502_19289_gb300 as P
@@ -620,19 +677,10 @@ def run_latency(args):
         run(w, base, False)   # warm-up
         plain = run(w, base, False)
         prof = run(w, base, True)
-        try:   # the same steps with every sweep loop driven from the host, then on the device
-            P.set_sweep_graphs(0)
-            host = run(w, base, False)
-            P.set_sweep_graphs(2)
-            dev = run(w, base, False)
-        finally:
-            P.set_sweep_graphs(1)
         ns = max(prof["steps"], 1)
         top = sorted(prof["classes"].items(), key=lambda kv: -kv[1]["ms"])[:5]
         res[name] = {"updates_per_s": plain["updates"] / plain["step_wall_s"], "steps": plain["steps"],
                      "step_ms": 1e3 * plain["step_wall_s"] / max(plain["steps"], 1),
-                     "step_ms_host_sweep_loop": 1e3 * host["step_wall_s"] / max(host["steps"], 1),
-                     "step_ms_device_sweep_loop": 1e3 * dev["step_wall_s"] / max(dev["steps"], 1),
                      "kernel_ms_per_step": prof["kernel_ms"] / ns,
                      "kernel_ms_per_step_by_class": {k: round(v["ms"] / ns, 4) for k, v in top},
                      "launches_per_step": prof["launches"] / ns,
@@ -882,9 +930,8 @@ def run_ours(args, rank, world, local_rank):
     if world > 1:
         import torch.distributed as dist
         dist.barrier()
-    # timed region: the library's default path (no per-launch events; each
-    # eigen-solve's sweeps run as one device-side graph); its launch and flop
-    # counters still accumulate
+    # timed region: the library's default path, no per-launch events; its launch
+    # and flop counters still accumulate
     P._check(P.lib.ctebd_profile(mps._h, 0), "profile")
     with Clocks(local_rank) as clk:
         for _ in range(args.steps):
@@ -904,12 +951,14 @@ def run_ours(args, rank, world, local_rank):
     res["steps_detail"] = step_f
     sw = np.concatenate(sweeps) if sweeps else np.zeros((0, 2))
     capped, capped_moved = mps.solver_stats()
-    res["jacobi_sweeps"] = {"splits": int(len(sw)), "cap": P.max_sweeps(),
+    direct = int((sw[:, 0] == 0).sum())   # direct and narrow splits make no sweeps
+    sw = sw[sw[:, 0] > 0]
+    res["jacobi_sweeps"] = {"splits": int(len(sw)), "splits_without_jacobi": direct, "cap": P.max_sweeps(),
                             "refinements_accepted_at_cap": capped, "their_max_moved_rel": capped_moved,
                             "pass1_mean": float(sw[:, 0].mean()) if len(sw) else 0.0,
                             "pass1_max": int(sw[:, 0].max()) if len(sw) else 0,
                             "pass2_mean": float(sw[:, 1].mean()) if len(sw) else 0.0,
-                            "pass2_max": int(sw[:, 1].max()) if len(sw) else 0}
+                            "pass2_max": int(sw[:, 1].max()) if len(sw) else 0} if len(sw) else None
     res["peaks"] = measure_compute_peaks(P, torch, device)
 
     # plain FP64 comparator on a sample of the next iteration's clusters
@@ -1143,12 +1192,13 @@ def main():
                          "with Q_max = kmax + 2 log2 chi: 6 lets k = 3..6 clusters form)")
     ap.add_argument("--plain-sample", type=int, default=2)
     ap.add_argument("--cpu-seconds", type=float, default=12.0)
-    ap.add_argument("--workload", default="cfg4", choices=["cfg4", "cfg2", "sketch-cfg4", "cfg5", "compare", "apply-traffic", "latency",
-                             "tebd", "shor"],
+    ap.add_argument("--workload", default="cfg4", choices=["cfg4", "cfg2", "sketch-cfg4", "cfg5", "compare", "apply-traffic",
+                             "bidiag-traffic", "latency", "tebd", "shor"],
                     help="cfg4: the headline (saturated chi=1024, full split); cfg2, sketch-cfg4: full vs "
                          "sketched split (cfg2, and cfg4's growing phase); "
                          "compare: FP32 path, FP64 mode and the plain FP64 path over the same iterations; "
-                         "apply-traffic: small case for the round update's DRAM traffic; latency: GPU-busy "
+                         "apply-traffic, bidiag-traffic: small cases for the round update's and the "
+                         "bidiagonalisation's DRAM traffic; latency: GPU-busy "
                          "fraction of the step on small configurations; cfg5: packed circuits, each "
                          "checked against its FP64-mode run; tebd: cluster-TEBD against standard "
                          "TEBD on the paper's generator; shor: the same on Shor's order-finding circuit")
@@ -1166,7 +1216,7 @@ def main():
                     help="cfg2 / sketch-cfg4: circuit depth (default: 50 / 30)")
     args = ap.parse_args()
     if args.n is None:
-        args.n = {"compare": 60, "apply-traffic": 24, "sketch-cfg4": 100}.get(args.workload, 500)
+        args.n = {"compare": 60, "apply-traffic": 24, "bidiag-traffic": 32, "sketch-cfg4": 100}.get(args.workload, 500)
     if args.chi is None:
         args.chi = {"tebd": 256, "shor": 256}.get(args.workload, 1024)
     if args.kmax is None:
@@ -1188,6 +1238,9 @@ def main():
         return
     if args.workload == "cfg5":
         run_cfg5(args)
+        return
+    if args.workload == "bidiag-traffic":
+        run_bidiag_traffic(args)
         return
     if args.workload == "apply-traffic":
         run_apply_traffic(args)
@@ -1258,8 +1311,7 @@ def main():
                 "launches": dom["launches"], "avg_launch_ms": dom["ms"] / max(dom["launches"], 1)}
     elif dom["flops"] > 0:
         achieved = dom["flops"] / (dom["ms"] / 1000.0) / 1e12
-        traffic, t_note = (apply_traffic_per_launch(dom["flops"] / max(dom["launches"], 1))
-                           if dom_name == "eig_apply" else (None, "no capture of this kernel"))
+        traffic, t_note = traffic_per_launch(dom_name, dom["flops"] / max(dom["launches"], 1))
         roof = {"kernel": dom_name, "bound": "alu", "achieved": achieved, "peak": alu_peak,
                 "unit": "TFLOP/s", "frac": achieved / alu_peak, "traffic": traffic,
                 "traffic_unit": "bytes per launch", "traffic_source": t_note,
@@ -1314,8 +1366,7 @@ def main():
         "kernels": {k: {"launches": int(v["launches"]), "ms": round(v["ms"], 3),
                         "share": round(v["ms"] / max(sum(x["ms"] for x in prof.values()), 1e-9), 4)}
                     for k, v in prof.items() if v["launches"] > 0},
-        "kernels_note": "per-launch CUDA events of one further iteration (host-driven sweeps); the timed "
-                        "iterations run the eigen-solve sweeps as device-side graphs without events",
+        "kernels_note": "per-launch CUDA events of one further iteration; the timed iterations run without events",
         "cpu_baseline": cpu,
         "e2e": {"value": units / wall if wall > 0 else 0.0, "unit": UNIT,
                 "h2d_bytes_per_step": int(res["h2d"] / max(args.steps, 1)),
@@ -1324,8 +1375,9 @@ def main():
         "clocks": clocks,
         "updates": units,
         "steps_detail": res["steps_detail"],
-        "jacobi_sweeps": res["jacobi_sweeps"],
     }
+    if res["jacobi_sweeps"]:   # splits that took the Gram matrix and Jacobi
+        line["jacobi_sweeps"] = res["jacobi_sweeps"]
     if "plain" in res and "error" in res["plain"]:
         line["plain_fp64"] = res["plain"]
     elif "plain" in res:
