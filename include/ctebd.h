@@ -315,12 +315,14 @@ int ctebd_set_sweep_graphs(int mode);
 /* Sweep cap of the Jacobi eigen-solves of the split (not in the paper; the
    solver of this implementation), process-wide, 1..1000 (default 60: the
    first pass takes about 10 sweeps at width 2048, the refinement pass up to
-   about 20 on steep spectra).  Full splits of the handle calls use a direct
-   solver without sweeps unless the cap is below 12 or the tensor-core policy
-   is 2; the Jacobi solver then takes them, with this cap.  A solve whose problems still make significant
-   rotations after n sweeps makes step / truncate_split / split2_noalloc return
-   CTEBD_ERR_NUMERIC (the state's sites of that iteration are then
-   undefined).  Errors: ARG. */
+   about 20 on steep spectra).  Full splits use a direct solver without sweeps,
+   except: with a cap below 12 the Jacobi solver takes them all, with that cap
+   (split2_noalloc too); in the handle calls, also with tensor-core policy 2, and
+   tall splits of wide clusters where the Gram matrix costs less or the direct
+   solver's scratch does not hold the rows.  A solve whose problems still make
+   significant rotations after n sweeps makes step / truncate_split /
+   split2_noalloc return CTEBD_ERR_NUMERIC (the state's sites of that iteration
+   are then undefined).  Errors: ARG. */
 int ctebd_set_max_sweeps(int n);
 
 /* The current sweep cap. */
