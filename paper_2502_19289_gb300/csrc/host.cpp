@@ -583,7 +583,7 @@ struct ctebd_mps {
 // at a quarter of it), and what a pool holds beyond a smaller share is given back.
 constexpr uint64_t kPoolKeep = (uint64_t)1 << 30;
 static std::mutex g_pools_lock;
-static std::vector<cudaMemPool_t> g_pools;
+static std::vector<cudaMemPool_t>& g_pools = *new std::vector<cudaMemPool_t>;   // outlives handles that go at exit
 static size_t g_pool_shares = 1;
 
 static cudaError_t pool_share(cudaMemPool_t p) {
