@@ -1833,9 +1833,11 @@ static bool use_direct(const ctebd_mps* m, int rows, int n) {
 // its trailing part twice per column, one problem after another, when the rows
 // of a level's problems do not fit the chip's shared memory side by side.  The
 // rule compares estimates in microseconds per level, for c problems:
-//   direct  c n (2 + 2e-6 m n),  3e-6 beyond 72 MB (L2);  FP64 c n (3 + 3.2e-5 m n);
-//           2.4 times the second term at 65 to 128 columns
-//   Gram    45 n + c (3.5e-6 n^3 + 0.55e-6 m n^2);  FP64 160 n + c (3e-4 n^3 + 1.2e-5 m n^2)
+//   direct  c n (2 + 2e-6 m n),  3e-6 beyond 96 MB (L2);  FP64 c n (3 + 3.2e-5 m n);
+//           twice the second term at 65 to 128 columns
+//   Gram    30 n + 0.015 n^2 + 0.25 m + c (3.5e-6 n^3 + 0.5e-6 m n^2);
+//           FP64 150 n + 0.6 m + c (3e-4 n^3 + 1.2e-5 m n^2);  n padded to whole
+//           block pairs
 // fitted to both sides of 124 shapes (16 to 2048 columns, 512 to 65536 rows, 1
 // to 16 problems, flat spectra).  Direct / Gram, ms of solver time per level:
 //   FP32  8192 x 512: 1 problem 6.9 / 27, 4: 24 / 29, 8: 47 / 36
@@ -1843,20 +1845,22 @@ static bool use_direct(const ctebd_mps* m, int rows, int n) {
 //         16384 x 1024: 1: 52 / 61, 4: 201 / 92;  65536 x 1024: 1: 244 / 76
 //         8192 x 2048: 2: 177 / 228;  16384 x 2048: 1: 217 / 199, 2: 430 / 289
 //   FP64  4096 x 128: 4: 26 / 21, 16: 100 / 38;  8192 x 512: 4: 269 / 363
-// The rule takes the faster side of all but six of them, there at most 1.27
-// times the other.  At m = 4 n and below the direct solver is the faster one.
+// The rule takes the slower side of five of them, by 1.07 to 1.27.  Whole
+// updates of 26 other shapes (chi 20 to 1024, decaying spectra among them):
+// never more than 1.02 times the better of the two.  At m = 4 n and below the
+// direct solver is the faster one.
 static bool gram_is_faster(const ctebd_mps* m, const Level& L, const std::vector<int>& tall) {
   const bool f64 = m->fp64;
-  double all = 0, direct = 0, gram = 0, widest = 0;
+  double all = 0, direct = 0, gram = 0, once = 0;
   for (int a : tall) {
-    const double mm = L.mm[a], n = L.nn[a], bytes = mm * n * (double)m->esz;
-    const double pass = (f64 ? 3.2e-5 : bytes <= 72e6 ? 2e-6 : 3e-6) * (n > 64 && n <= 128 ? 2.4 : 1.0);
+    const double mm = L.mm[a], n = L.nn[a], np = L.npad[a], bytes = mm * n * (double)m->esz;
+    const double pass = (f64 ? 3.2e-5 : bytes <= 96e6 ? 2e-6 : 3e-6) * (n > 64 && n <= 128 ? 2 : 1);
     direct += n * ((f64 ? 3 : 2) + pass * mm * n);
-    gram += f64 ? 3e-4 * n * n * n + 1.2e-5 * mm * n * n : 3.5e-6 * n * n * n + 0.55e-6 * mm * n * n;
+    gram += f64 ? (3e-4 * np + 1.2e-5 * mm) * np * np : (3.5e-6 * np + 0.5e-6 * mm) * np * np;
+    once = std::max(once, f64 ? 150 * np + 0.6 * mm : (30 + 0.015 * np) * np + 0.25 * mm);
     all += bytes;
-    widest = std::max(widest, n);
   }
-  return all > m->n_sm * 226e3 && direct > gram + (f64 ? 160 : 45) * widest;
+  return all > m->n_sm * 226e3 && direct > gram + once;
 }
 
 // pass 1 (+ FP32 pass 2) for a selection: Gram of Z, eigen-solve, V, weights, select
