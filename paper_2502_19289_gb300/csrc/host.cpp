@@ -586,20 +586,20 @@ static std::mutex g_pools_lock;
 static std::vector<cudaMemPool_t>& g_pools = *new std::vector<cudaMemPool_t>;   // outlives handles that go at exit
 static size_t g_pool_shares = 1;
 
-static cudaError_t pool_share(cudaMemPool_t p) {
+static cudaError_t pool_share(cudaMemPool_t p, bool trim) {
   uint64_t keep = kPoolKeep / g_pool_shares;
   const cudaError_t e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-  return e != cudaSuccess ? e : cudaMemPoolTrimTo(p, keep);
+  return e != cudaSuccess || !trim ? e : cudaMemPoolTrimTo(p, keep);
 }
 static cudaError_t pool_open(cudaMemPool_t* p, const cudaMemPoolProps& props) {
   cudaError_t e = cudaMemPoolCreate(p, &props);
   if (e != cudaSuccess) { *p = nullptr; return e; }
   std::lock_guard<std::mutex> lock(g_pools_lock);
   g_pools.push_back(*p);
-  if (g_pools.size() <= g_pool_shares) return pool_share(*p);
+  if (g_pools.size() <= g_pool_shares) return pool_share(*p, false);
   g_pool_shares *= 2;
   for (cudaMemPool_t q : g_pools)
-    if (cudaError_t r = pool_share(q)) e = r;
+    if (cudaError_t r = pool_share(q, q != *p)) e = r;
   return e;
 }
 static void pool_close(cudaMemPool_t p) {
@@ -608,7 +608,7 @@ static void pool_close(cudaMemPool_t p) {
     g_pools.erase(std::find(g_pools.begin(), g_pools.end(), p));
     if (g_pool_shares > 1 && g_pools.size() <= g_pool_shares / 4) {
       g_pool_shares /= 2;
-      for (cudaMemPool_t q : g_pools) pool_share(q);
+      for (cudaMemPool_t q : g_pools) pool_share(q, false);
     }
   }
   cudaMemPoolDestroy(p);
